@@ -50,6 +50,14 @@ constexpr int kTile = 8;   // active-list entries per thread per scan tile
 constexpr int kExpand = 4; // staged frontier vertices per thread per expansion round
 constexpr int kIlp = 8;    // arcs per lane in flight
 constexpr int kTake = 32;  // queue items per chunk of a warp's share
+// Crossing vertices a warp stages before it pushes them together: an
+// iteration's maximum (kWarp * kIlp) on top of what it may leave waiting
+// (kHold). The sampling kernel's shared memory holds fewer, so it also pushes
+// inside an iteration.
+constexpr int kHold = kWarp;
+constexpr int kStage = kWarp * kIlp + kHold;
+constexpr int kStageS = 128;
+constexpr int kPrefetchSlices = 256;  // appends of at most this many slices prefetch their arcs
 constexpr int kLenShift = 40;  // item = first arc | length << 40
 constexpr unsigned long long kArcMask = (1ull << kLenShift) - 1;
 // barrier word: arrivals in bits 0..30, the phase's queue appends in bits
@@ -67,8 +75,7 @@ __shared__ unsigned long long s_app;
 __shared__ int s_abort;
 
 struct Shared {
-  int excl[kWarps][kWarp];
-  long long a0[kWarps][kWarp];
+  long long delta[kWarps][kWarp];  // passes: the batch's arc map (ArcMap)
   union {
     unsigned long long lq[kWarps][kLocalQueueMax];  // passes: the warps' local queues
     int stage[kBlock * kTile];                      // scans (local queues are empty): frontier ids
@@ -107,15 +114,20 @@ struct Shared {
   unsigned tail_gen;  // tail episodes begun (thread 0 of every CTA)
 };
 
+struct SharedN : Shared {
+  int xs[kWarps][kStage];  // passes: crossing vertices waiting to be pushed
+};
+
 // Sampling keeps the vertex of each local-queue entry beside it (a spilled
 // entry's vertex is traversed a pass later, which its stamp must say) and the
 // warps' head counts.
 struct SharedS : Shared {
+  int xs[kWarps][kStageS];
   int lqv[kWarps][kLocalQueueMax];
   unsigned long long heads[kWarps];
 };
 template <bool kSample>
-using ShT = std::conditional_t<kSample, SharedS, Shared>;
+using ShT = std::conditional_t<kSample, SharedS, SharedN>;
 
 // Records the first error and makes every CTA leave at its next barrier (or,
 // parked during a tail episode, at once).
@@ -124,6 +136,19 @@ __device__ __forceinline__ void raise_status(const PeelArgs& a, int code) {
   for (int i = 0; i < 3; i++) atomicOr(&a.ctl->bar_ring[i].v, kAbort);
   atomicOr(&a.ctl->tail_word, kAbort);
   s_abort = 1;
+}
+
+// Slices of an arc range: a list holds fewer than 2^31 arcs and a slice at most
+// 2^20, so the division is a 32-bit one (the 64-bit one by a run-time divisor
+// is a long dependent sequence in the middle of a crossing's chain).
+__device__ __forceinline__ int slices_of(const PeelArgs& a, long long e0, long long e1) {
+  return (int)(((unsigned)(e1 - e0) + (unsigned)a.slice - 1u) / (unsigned)a.slice);
+}
+
+// Starts the read of an appended slice's first line: the next phase reads it
+// from L2 instead of DRAM. Only for appends small enough to stay in L2.
+__device__ __forceinline__ void prefetch_arcs(const PeelArgs& a, long long arc) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(a.adj + arc));
 }
 
 __device__ __forceinline__ unsigned long long make_item(long long a0, long long len) {
@@ -246,7 +271,7 @@ __device__ void append_recount(const PeelArgs& a, RoundRec* R, bool flag, int v,
 // Returns false when a status was raised before the barrier completed, or
 // when the wait gave up. With R, thread 0 then also reads R's other counters
 // (and the sampling miss flag) into sh.po for the whole CTA.
-__device__ bool grid_barrier(const PeelArgs& a, Shared& sh, unsigned long long& gen,
+__device__ bool grid_barrier(const PeelArgs& a, Shared& sh, unsigned& gen,
                              const RoundRec* R = nullptr) {
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -468,7 +493,7 @@ __device__ ScanOut scan_range(const PeelArgs& a, Shared& sh, RoundRec* R, unsign
         }
       }
 #pragma unroll
-      for (int k = 0; k < kExpand; k++) nsl += (int)((e1[k] - e0[k] + a.slice - 1) / a.slice);
+      for (int k = 0; k < kExpand; k++) nsl += slices_of(a, e0[k], e1[k]);
       int ntot;
       const int exs = block_excl_scan(sh, nsl, &ntot);
       if (tid == 0) {
@@ -485,8 +510,10 @@ __device__ ScanOut scan_range(const PeelArgs& a, Shared& sh, RoundRec* R, unsign
         unsigned long long pq = sh.base_q + exs;
 #pragma unroll
         for (int k = 0; k < kExpand; k++)
-          for (long long s0 = e0[k]; s0 < e1[k]; s0 += a.slice)
+          for (long long s0 = e0[k]; s0 < e1[k]; s0 += a.slice) {
             a.Q[pq++] = make_item(s0, min((long long)a.slice, e1[k] - s0));
+            if (ntot <= kPrefetchSlices) prefetch_arcs(a, s0);
+          }
       }
       __syncthreads();
     }
@@ -553,7 +580,10 @@ __device__ __forceinline__ void append_ranges(const PeelArgs& a, const PassCtx& 
   if constexpr (kCoop) {
     write_slices(a, e0, e1, cnt, p, lane);
   } else {
-    for (long long s0 = e0; s0 < e1 && cnt > 0; s0 += a.slice) a.Q[p++] = make_item(s0, min((long long)a.slice, e1 - s0));
+    for (long long s0 = e0; s0 < e1 && cnt > 0; s0 += a.slice) {
+      a.Q[p++] = make_item(s0, min((long long)a.slice, e1 - s0));
+      if (tot <= kPrefetchSlices) prefetch_arcs(a, s0);
+    }
   }
 }
 
@@ -568,9 +598,9 @@ __device__ __forceinline__ void push_crossed(const PeelArgs& a, ShT<kSample>& sh
   if (flag) {
     e0 = __ldcs(a.off + u);
     e1 = __ldcs(a.off + u + 1);
-    nsl = (int)((e1 - e0 + a.slice - 1) / a.slice);
+    nsl = slices_of(a, e0, e1);
     // its first adjacency line is read next, here or by another warp
-    if (e1 > e0) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.adj + e0));
+    if (e1 > e0) prefetch_arcs(a, e0);
   }
   const bool one = flag && nsl == 1;
   const unsigned om = __ballot_sync(kFull, one);
@@ -590,6 +620,63 @@ __device__ __forceinline__ void push_crossed(const PeelArgs& a, ShT<kSample>& sh
   append_ranges(a, pc, (flag && !local) ? nsl : 0, e0, e1, lane);
 }
 
+// Pushes the nx vertices staged in sh.xs[warp], 32 at a time. Warp-collective.
+// A push is a chain of its own (the vertices' offsets from DRAM, the append's
+// atomic on the one word that every warp appends to); pushing slot by slot of
+// an iteration walked it up to kIlp times and sent as many atomics. Staged and
+// pushed once per iteration at most: R-MAT 24 16.19 -> 14.86 ms, R-MAT 20 5.00
+// -> 4.71, kNN 5.51 -> 4.18, a kNN graph peeled by one narrow wave 50.4 ->
+// 35.5 (together with the arc map, the 32-bit divisions and the prefetch of
+// appended slices).
+template <bool kSample = false>
+__device__ __forceinline__ void push_staged(const PeelArgs& a, ShT<kSample>& sh, const PassCtx& pc, int nx, int warp,
+                                            int lane) {
+  __syncwarp();
+  for (int b = 0; b < nx; b += kWarp) {
+    const bool f = b + lane < nx;
+    push_crossed<kSample>(a, sh, pc, f, f ? sh.xs[warp][b + lane] : 0, warp, lane);
+  }
+  __syncwarp();
+}
+
+// Spreads the arcs of a batch of items (lane i < c holds an item of len > 0
+// arcs from a0) over the warp: arc position j of the batch belongs to lane
+// j % 32 of window j / 32. Which item a position falls in comes from the bit
+// mask of the items that start inside its window (one warp reduction, then a
+// population count), not from a search: the map is on the dependent chain of
+// every short pass, where one warp issues it with nothing to hide it behind.
+struct ArcMap {
+  const long long* delta;  // shared memory: item i's first arc minus its first position
+  int start;               // first position of this lane's item (past every window when it has none)
+  int total;
+  // the first arc of the window at position base + this lane; before: items
+  // that start ahead of the window (kept by the caller across windows)
+  __device__ __forceinline__ long long arc(int base, int lane, int& before) const {
+    const unsigned d = (unsigned)(start - base);
+    const unsigned m = __reduce_or_sync(kFull, d < (unsigned)kWarp ? 1u << d : 0u);
+    const int idx = before + __popc(m & (lanemask_lt() | (1u << lane))) - 1;
+    before += __popc(m);
+    return delta[idx] + base + lane;
+  }
+};
+
+// Warp-collective. An item outside [0, m) raises ST_NOT_SIMPLE and leaves the
+// batch empty, so no arc past the adjacency array is ever read.
+__device__ __forceinline__ ArcMap map_items(const PeelArgs& a, Shared& sh, unsigned long long item, int c, int warp,
+                                            int lane) {
+  const long long a0 = lane < c ? (long long)(item & kArcMask) : 0;
+  const int len = lane < c ? (int)(item >> kLenShift) : 0;
+  const int incl = warp_incl_scan(len, lane);
+  sh.delta[warp][lane] = a0 - (incl - len);
+  ArcMap mp{sh.delta[warp], len > 0 ? incl - len : INT_MAX, __shfl_sync(kFull, incl, 31)};
+  if (__any_sync(kFull, a0 + len > a.m)) {
+    if (lane == 0) raise_status(a, ST_NOT_SIMPLE);
+    mp.total = 0;
+  }
+  __syncwarp();
+  return mp;
+}
+
 // Arcs of the items held by lanes < c, spread evenly over the warp.
 // With sampling (kSample), d~ is always read first: a neighbour in sample
 // mode (d~ < 0) is not decremented but tosses the arc's coin, and its mu-th
@@ -598,36 +685,25 @@ template <bool kWin, bool kSample = false, bool kCombine = false>
 __device__ void process_items(const PeelArgs& a, ShT<kSample>& sh, const PassCtx& pc, unsigned long long item,
                               int c, int warp, int lane) {
   const int t = pc.t;
-  const long long a0 = lane < c ? (long long)(item & kArcMask) : 0;
-  const int len = lane < c ? (int)(item >> kLenShift) : 0;
-  const int incl = warp_incl_scan(len, lane);
-  const int total = __shfl_sync(kFull, incl, 31);
-  sh.excl[warp][lane] = incl - len;
-  sh.a0[warp][lane] = a0;
-  __syncwarp();
-  const int* excl = sh.excl[warp];
+  const ArcMap mp = map_items(a, sh, item, c, warp, lane);
+  const int total = mp.total;
   int ndec = 0;
   unsigned nheads = 0;
+  int nx = 0;             // crossing vertices staged (warp-uniform)
+  int before = 0;         // items that start ahead of the window
   for (int base = 0; base < total; base += kWarp * kIlp) {
     int u[kIlp];
-    int j = base + lane;
-    int lo = 0, hi = c;  // last item whose first arc is <= j
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (excl[mid] <= j) lo = mid + 1;
-      else hi = mid;
-    }
-    int idx = lo > 0 ? lo - 1 : 0;
-    const int idx0 = idx;
+    const int before0 = before;
 #pragma unroll
-    for (int q = 0; q < kIlp; q++, j += kWarp) {
+    for (int q = 0; q < kIlp; q++) {
       u[q] = -1;
-      if (j < total) {
-        while (idx + 1 < c && excl[idx + 1] <= j) idx++;
-        const long long arc = sh.a0[warp][idx] + (j - excl[idx]);
-        const int x = arc < a.m ? ld_stream_s32(a.adj + arc) : -1;
-        if ((unsigned)x < (unsigned)a.n) u[q] = x;
-        else raise_status(a, ST_NOT_SIMPLE);
+      if (base + q * kWarp < total) {
+        const long long arc = mp.arc(base + q * kWarp, lane, before);
+        if (base + q * kWarp + lane < total) {
+          const int x = ld_stream_s32(a.adj + arc);
+          if ((unsigned)x < (unsigned)a.n) u[q] = x;
+          else raise_status(a, ST_NOT_SIMPLE);
+        }
       }
     }
     // Reading d~ first spares the atomics on neighbours at or below the
@@ -647,20 +723,20 @@ __device__ void process_items(const PeelArgs& a, ShT<kSample>& sh, const PassCtx
     }
     unsigned cross = 0, enter = 0, bag = 0;
     if constexpr (kSample) {
-      int ix = idx0;
+      int before1 = before0;
 #pragma unroll
-      for (int q = 0; q < kIlp; q++)
+      for (int q = 0; q < kIlp; q++) {
+        if (base + q * kWarp >= total) continue;
+        const long long arc = mp.arc(base + q * kWarp, lane, before1);
         if (u[q] >= 0 && dq[q] < 0) {
           // sample mode: one coin of probability mu / ((1 - r) D) per arc,
           // drawn from the arc's index
-          const int jq = base + lane + q * kWarp;
-          while (ix + 1 < c && excl[ix + 1] <= jq) ix++;
-          const long long arc = sh.a0[warp][ix] + (jq - excl[ix]);
           if (coin_head(philox_coin((unsigned long long)arc, a.seed), -1 - dq[q], a.coin_lim)) {
             nheads++;
             if (atomicAdd(a.scnt + u[q], 1) == a.mu - 1) bag |= 1u << q;
           }
         }
+      }
     }
 #pragma unroll
     for (int q = 0; q < kIlp; q++)
@@ -712,13 +788,22 @@ __device__ void process_items(const PeelArgs& a, ShT<kSample>& sh, const PassCtx
 #pragma unroll
       for (int q = 0; q < kIlp; q++) {
         const bool f = (cross >> q) & 1u;
-        if (f) a.core[u[q]] = pc.val;
-        if (__any_sync(kFull, f)) push_crossed<kSample>(a, sh, pc, f, u[q], warp, lane);
+        const unsigned fm = __ballot_sync(kFull, f);
+        if (f) {
+          a.core[u[q]] = pc.val;
+          sh.xs[warp][nx + __popc(fm & lanemask_lt())] = u[q];
+        }
+        nx += __popc(fm);
+        if (kSample && nx > kStageS - kWarp) {
+          push_staged<kSample>(a, sh, pc, nx, warp, lane);
+          nx = 0;
+        }
       }
-      if (a.threshold) {
-        const int nc = warp_sum(__popc(cross));
-        if (lane == 0) sh.ncross[warp] += nc;
-      }
+    }
+    if (nx > (base + kWarp * kIlp < total ? kHold : 0)) {
+      push_staged<kSample>(a, sh, pc, nx, warp, lane);
+      if (a.threshold && lane == 0) sh.ncross[warp] += nx;
+      nx = 0;
     }
   }
   if (a.trace) {
@@ -778,6 +863,26 @@ __device__ void drain_local(const PeelArgs& a, ShT<kSample>& sh, const PassCtx& 
   }
 }
 
+// Warp gw's contiguous share [b, e) of the queue range [qb, qe) over nw warps:
+// len / nw items, one more for the first len % nw warps (32-bit division
+// unless the range is longer: a 64-bit one is a long dependent sequence).
+__device__ __forceinline__ unsigned long long warp_share(unsigned long long qb, unsigned long long qe, unsigned gw,
+                                                         unsigned nw, unsigned long long* e) {
+  const unsigned long long len = qe - qb;
+  unsigned long long share;
+  unsigned rem;
+  if (len >> 32) {
+    share = len / nw;
+    rem = (unsigned)(len % nw);
+  } else {
+    share = (unsigned)len / nw;
+    rem = (unsigned)len - (unsigned)share * nw;
+  }
+  const unsigned long long b = qb + gw * share + min(gw, rem);
+  *e = b + share + (gw < rem ? 1 : 0);
+  return b;
+}
+
 // One subround: the queue range [qb, qe) is processed once by `nctas` CTAs
 // (the grid, or CTA 0 alone in tail mode), this one being number `cta`. Warp
 // gw takes its own contiguous share (len / warps items, one more for the
@@ -787,11 +892,9 @@ template <bool kWin, bool kSample = false, bool kCombine = false>
 __device__ void run_pass(const PeelArgs& a, ShT<kSample>& sh, const PassCtx& pc, unsigned long long qb,
                          unsigned long long qe, int cta, int nctas) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned long long gw = (unsigned long long)cta * kWarps + warp;
-  const unsigned long long nw = (unsigned long long)nctas * kWarps;
-  const unsigned long long len = qe - qb, share = len / nw, rem = len % nw;
-  const unsigned long long b = qb + gw * share + (gw < rem ? gw : rem);
-  const unsigned long long e = b + share + (gw < rem ? 1 : 0);
+  const unsigned gw = (unsigned)cta * kWarps + warp, nw = (unsigned)nctas * kWarps;
+  unsigned long long e;
+  const unsigned long long b = warp_share(qb, qe, gw, nw, &e);
   for (unsigned long long pos = b; pos < e; pos += kTake) {
     const int c = (int)min((unsigned long long)kTake, e - pos);
     const unsigned long long item = lane < c ? ld_once_u64(a.Q + pos + lane, l2_evict_first_policy()) : 0;
@@ -814,33 +917,21 @@ template <bool kTouched>
 __device__ void hist_items(const PeelArgs& a, Shared& sh, const PassCtx& pc, unsigned long long item, int c,
                            int warp, int lane) {
   const int t = pc.t;
-  const long long a0 = lane < c ? (long long)(item & kArcMask) : 0;
-  const int len = lane < c ? (int)(item >> kLenShift) : 0;
-  const int incl = warp_incl_scan(len, lane);
-  const int total = __shfl_sync(kFull, incl, 31);
-  sh.excl[warp][lane] = incl - len;
-  sh.a0[warp][lane] = a0;
-  __syncwarp();
-  const int* excl = sh.excl[warp];
+  const ArcMap mp = map_items(a, sh, item, c, warp, lane);
+  const int total = mp.total;
+  int before = 0;
   for (int base = 0; base < total; base += kWarp * kIlp) {
     int u[kIlp];
-    int j = base + lane;
-    int lo = 0, hi = c;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (excl[mid] <= j) lo = mid + 1;
-      else hi = mid;
-    }
-    int idx = lo > 0 ? lo - 1 : 0;
 #pragma unroll
-    for (int q = 0; q < kIlp; q++, j += kWarp) {
+    for (int q = 0; q < kIlp; q++) {
       u[q] = -1;
-      if (j < total) {
-        while (idx + 1 < c && excl[idx + 1] <= j) idx++;
-        const long long arc = sh.a0[warp][idx] + (j - excl[idx]);
-        const int x = arc < a.m ? ld_stream_s32(a.adj + arc) : -1;
-        if ((unsigned)x < (unsigned)a.n) u[q] = x;
-        else raise_status(a, ST_NOT_SIMPLE);
+      if (base + q * kWarp < total) {
+        const long long arc = mp.arc(base + q * kWarp, lane, before);
+        if (base + q * kWarp + lane < total) {
+          const int x = ld_stream_s32(a.adj + arc);
+          if ((unsigned)x < (unsigned)a.n) u[q] = x;
+          else raise_status(a, ST_NOT_SIMPLE);
+        }
       }
     }
     int dq[kIlp];
@@ -878,11 +969,9 @@ template <bool kTouched>
 __device__ void run_hist(const PeelArgs& a, Shared& sh, const PassCtx& pc, unsigned long long qb,
                          unsigned long long qe) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned long long gw = (unsigned long long)blockIdx.x * kWarps + warp;
-  const unsigned long long nw = (unsigned long long)gridDim.x * kWarps;
-  const unsigned long long len = qe - qb, share = len / nw, rem = len % nw;
-  const unsigned long long b = qb + gw * share + (gw < rem ? gw : rem);
-  const unsigned long long e = b + share + (gw < rem ? 1 : 0);
+  const unsigned gw = blockIdx.x * kWarps + warp, nw = gridDim.x * kWarps;
+  unsigned long long e;
+  const unsigned long long b = warp_share(qb, qe, gw, nw, &e);
   for (unsigned long long pos = b; pos < e; pos += kTake) {
     const int c = (int)min((unsigned long long)kTake, e - pos);
     const unsigned long long item = lane < c ? ld_once_u64(a.Q + pos + lane, l2_evict_first_policy()) : 0;
@@ -916,7 +1005,7 @@ __device__ void run_apply(const PeelArgs& a, const PassCtx& pc, const int* list,
           a.core[u] = pc.val;
           e0 = a.off[u];
           e1 = a.off[u + 1];
-          nsl = (int)((e1 - e0 + a.slice - 1) / a.slice);
+          nsl = slices_of(a, e0, e1);
         }
       } else {
         raise_status(a, ST_CAPACITY);
@@ -1018,7 +1107,7 @@ __device__ void run_recount_apply(const PeelArgs& a, const PassCtx& pc, unsigned
     }
     const unsigned jm = __ballot_sync(kFull, join);
     if (jm && lane == 0) atomicAdd(&pc.R->found, (unsigned long long)__popc(jm));
-    const int nsl = join ? (int)((e1 - e0 + a.slice - 1) / a.slice) : 0;
+    const int nsl = join ? slices_of(a, e0, e1) : 0;
     append_ranges<true>(a, pc, nsl, e0, e1, lane);
   }
   kmin = warp_min(kmin);
@@ -1049,7 +1138,7 @@ __global__ void __launch_bounds__(kBlock, 2) peel_bsp(PeelArgs a) {
     if constexpr (kSample) sh.heads[warp] = 0;
   }
   // grid barriers taken; grid phase g uses RoundRec g % 3 and barrier word g % 3
-  unsigned long long gen = 0;
+  unsigned gen = 0;
   // Tail mode (the plain schedule only): a phase whose range is small runs on
   // CTA 0 alone and ends at a CTA barrier; its counters live in the CTA's own
   // ring of records (tail phase s uses sh.tring[s % 3]).
@@ -1086,9 +1175,15 @@ __global__ void __launch_bounds__(kBlock, 2) peel_bsp(PeelArgs a) {
       a.ctl->bar_ring[r].v = 0;
     }
   };
+  // CTAs of a scan over len entries (a list holds at most n < 2^31), and the
+  // start of CTA b's part: 32-bit arithmetic, on every scan's dependent chain
   auto nscan_of = [&](long long len) {
-    long long ns = (len + a.scan_min - 1) / a.scan_min;
-    return ns < 1 ? 1ll : (ns > (long long)gridDim.x ? (long long)gridDim.x : ns);
+    const unsigned ns = ((unsigned)len + (unsigned)a.scan_min - 1) / (unsigned)a.scan_min;
+    return (long long)(ns < 1 ? 1u : min(ns, gridDim.x));
+  };
+  auto scan_lo = [&](long long len, long long nscan, unsigned b) {
+    const unsigned per = ((unsigned)len + (unsigned)nscan - 1) / (unsigned)nscan;
+    return min(len, (long long)per * b);
   };
   auto free_list = [&](const int* x, const int* y) -> int* {
     return (x != a.A0 && y != a.A0) ? a.A0 : ((x != a.A1 && y != a.A1) ? a.A1 : a.A2);
@@ -1267,7 +1362,7 @@ __global__ void __launch_bounds__(kBlock, 2) peel_bsp(PeelArgs a) {
       int* Aov = rebuild ? (Acur ? const_cast<int*>(Acur) : free_list(Aout, Aover)) : nullptr;
       long long nscan = solo ? 1 : nscan_of(lin);
       if (blockIdx.x < nscan) {
-        const long long lo = lin * blockIdx.x / nscan, hi = lin * (blockIdx.x + 1) / nscan;
+        const long long lo = scan_lo(lin, nscan, blockIdx.x), hi = scan_lo(lin, nscan, blockIdx.x + 1);
         const ScanOut o = a.threshold ? scan_range(a, sh, R, qend, Ain, Aout, lo, hi, tk, tk, true, 0, 1)
                           : rebuild  ? scan_range(a, sh, R, qend, Ain, Aout, lo, hi, tk, tk, false, -1, -1, Aov,
                                                   tk + W)
@@ -1320,7 +1415,7 @@ __global__ void __launch_bounds__(kBlock, 2) peel_bsp(PeelArgs a) {
         R = rec();
         nscan = solo ? 1 : nscan_of(la);
         if (blockIdx.x < nscan) {
-          const long long lo = la * blockIdx.x / nscan, hi = la * (blockIdx.x + 1) / nscan;
+          const long long lo = scan_lo(la, nscan, blockIdx.x), hi = scan_lo(la, nscan, blockIdx.x + 1);
           const ScanOut o = scan_range(a, sh, R, qend, Acur, nullptr, lo, hi, INT_MAX, t);
           if (tid == 0 && o.found) atomicAdd(&R->found, o.found);
         }
@@ -1534,7 +1629,7 @@ __global__ void __launch_bounds__(kBlock, 2) peel_bsp(PeelArgs a) {
       const long long lin = la;
       const long long nscan = nscan_of(lin);
       if (blockIdx.x < nscan) {
-        const long long lo = lin * blockIdx.x / nscan, hi = lin * (blockIdx.x + 1) / nscan;
+        const long long lo = scan_lo(lin, nscan, blockIdx.x), hi = scan_lo(lin, nscan, blockIdx.x + 1);
         const ScanOut o = scan_range<true>(a, sh, R, qend, Acur, Aout, lo, hi, tk, tk, false, -1, -1, nullptr,
                                            INT_MAX, (int)passes);
         if (tid == 0) {
@@ -1630,7 +1725,7 @@ __global__ void __launch_bounds__(kBlock, 2) barrier_probe(PeelArgs a, int iters
     s_app = 0;
     s_abort = 0;
   }
-  unsigned long long gen = 0;
+  unsigned gen = 0;
   __syncthreads();
   const uint64_t t0 = globaltimer_ns();
   for (int i = 0; i < iters; i++) {
