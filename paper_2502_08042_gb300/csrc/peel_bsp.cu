@@ -385,64 +385,84 @@ __device__ ScanOut scan_range(const PeelArgs& a, Shared& sh, RoundRec* R, unsign
       const long long i = tile + (long long)q * kBlock + tid;
       v[q] = i < hi ? (Ain ? ld_once_s32(Ain + i, l2_evict_first_policy()) : (int)i) : -1;
     }
+    // the d~ of the tile's entries, every load issued before any is used (a
+    // check that can branch between two loads makes each wait for the one
+    // before); failed checks are raised once per tile
+    int d[kTile];
+    bool bad = false;
+    if (Ain) {
+#pragma unroll
+      for (int q = 0; q < kTile; q++) {
+        const bool in = (unsigned)v[q] < (unsigned)a.n;
+        bad |= !in && tile + (long long)q * kBlock + tid < hi;
+        if (!in) v[q] = -1;
+        d[q] = in ? __ldcg(a.deg + v[q]) : 0;
+      }
+    } else {
+      constexpr int kPair = 4;  // offset pairs in flight per thread
+#pragma unroll
+      for (int q0 = 0; q0 < kTile; q0 += kPair) {
+        long long o0[kPair], o1[kPair];
+#pragma unroll
+        for (int q = 0; q < kPair; q++) {
+          const int x = v[q0 + q];
+          o0[q] = x >= 0 ? a.off[x] : 0;
+          o1[q] = x >= 0 ? a.off[x + 1] : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < kPair; q++) {
+          const int x = v[q0 + q];
+          d[q0 + q] = 0;
+          if (x < 0) continue;
+          if (o0[q] < 0 || o1[q] < o0[q] || o1[q] > a.m || o1[q] - o0[q] >= a.n) {
+            // malformed offsets: no arc of x is ever read; it is neither kept
+            // nor expanded and takes level 0
+            bad = true;
+            a.deg[x] = 0;
+            a.core[x] = 0;
+            v[q0 + q] = -1;
+          } else {
+            d[q0 + q] = (int)(o1[q] - o0[q]);
+            a.deg[x] = d[q0 + q];
+          }
+        }
+      }
+    }
+    if (bad) raise_status(a, ST_NOT_SIMPLE);
 #pragma unroll
     for (int q = 0; q < kTile; q++) {
       const int x = v[q];
-      if (x < 0 && tile + (long long)q * kBlock + tid >= hi) continue;
-      if ((unsigned)x >= (unsigned)a.n) {
-        raise_status(a, ST_NOT_SIMPLE);
-        v[q] = -1;
-        continue;
-      }
-      int d;
-      if (!Ain) {
-        const long long e0 = a.off[x], e1 = a.off[x + 1];
-        if (e0 < 0 || e1 < e0 || e1 > a.m || e1 - e0 >= a.n) {
-          raise_status(a, ST_NOT_SIMPLE);  // malformed offsets: no arc of x is ever read
-          d = -1;
-        } else {
-          d = (int)(e1 - e0);
-        }
-        a.deg[x] = d < 0 ? 0 : d;
-        if (d < 0) {
-          // a malformed vertex is neither kept nor expanded; it takes level 0
-          a.core[x] = 0;
-          v[q] = -1;
-          continue;
-        }
-        if constexpr (kSample) {
+      if (x < 0) continue;
+      const int dx = d[q];
+      if constexpr (kSample) {
+        if (!Ain) {
           a.stamp[x] = INT_MAX;
           a.scnt[x] = 0;
           a.racc[x] = 0;
           a.rst[x] = 0;
-          if (d > 0 && (long long)d > a.sthreshold) {  // InitSampler(v, 0)
-            a.deg[x] = -1 - d;
+          if (dx > 0 && (long long)dx > a.sthreshold) {  // InitSampler(v, 0)
+            a.deg[x] = -1 - dx;
             nsampled++;
             keep |= 1u << q;
-            dmin = min(dmin, sample_key(d, 0, a.mu));
+            dmin = min(dmin, sample_key(dx, 0, a.mu));
             continue;
           }
-        }
-      } else {
-        d = __ldcg(a.deg + x);
-        if constexpr (kSample) {
-          if (d < 0) {  // in sample mode: validate at level take_at
-            const int D = -1 - d, cnt = __ldcg(a.scnt + x);
-            keep |= 1u << q;
-            if (sample_safe(D, cnt, take_at, a.mu)) dmin = min(dmin, sample_key(D, cnt, a.mu));
-            else rec |= 1u << q;
-            continue;
-          }
+        } else if (dx < 0) {  // in sample mode: validate at level take_at
+          const int D = -1 - dx, cnt = __ldcg(a.scnt + x);
+          keep |= 1u << q;
+          if (sample_safe(D, cnt, take_at, a.mu)) dmin = min(dmin, sample_key(D, cnt, a.mu));
+          else rec |= 1u << q;
+          continue;
         }
       }
-      if (d > keep_above) {
-        if (d >= over_from) over |= 1u << q;
+      if (dx > keep_above) {
+        if (dx >= over_from) over |= 1u << q;
         else keep |= 1u << q;
-        dmin = min(dmin, d);
+        dmin = min(dmin, dx);
         if (keep_val >= 0) a.core[x] = keep_val;
       }
-      if (take_le ? d <= take_at : d == take_at) {
-        if (!Ain && d == 0) {
+      if (take_le ? dx <= take_at : dx == take_at) {
+        if (!Ain && dx == 0) {
           a.core[x] = take_val;  // first scan: no arcs, nothing to expand
           direct++;
         } else {
@@ -677,6 +697,21 @@ __device__ __forceinline__ ArcMap map_items(const PeelArgs& a, Shared& sh, unsig
   return mp;
 }
 
+// Checks the ids an iteration read (slot q of a lane holds one when
+// q * 32 < left): one outside [0, n) raises ST_NOT_SIMPLE and becomes -1. Apart
+// from the loads: a check that can branch between two of them makes each wait
+// for the one before.
+__device__ __forceinline__ void check_ids(const PeelArgs& a, int* u, int left) {
+  bool bad = false;
+#pragma unroll
+  for (int q = 0; q < kIlp; q++) {
+    const bool b = q * kWarp < left && (unsigned)u[q] >= (unsigned)a.n;
+    bad |= b;
+    if (b) u[q] = -1;
+  }
+  if (bad) raise_status(a, ST_NOT_SIMPLE);
+}
+
 // Arcs of the items held by lanes < c, spread evenly over the warp.
 // With sampling (kSample), d~ is always read first: a neighbour in sample
 // mode (d~ < 0) is not decremented but tosses the arc's coin, and its mu-th
@@ -699,13 +734,10 @@ __device__ void process_items(const PeelArgs& a, ShT<kSample>& sh, const PassCtx
       u[q] = -1;
       if (base + q * kWarp < total) {
         const long long arc = mp.arc(base + q * kWarp, lane, before);
-        if (base + q * kWarp + lane < total) {
-          const int x = ld_stream_s32(a.adj + arc);
-          if ((unsigned)x < (unsigned)a.n) u[q] = x;
-          else raise_status(a, ST_NOT_SIMPLE);
-        }
+        if (base + q * kWarp + lane < total) u[q] = ld_stream_s32(a.adj + arc);
       }
     }
+    check_ids(a, u, total - base - lane);
     // Reading d~ first spares the atomics on neighbours at or below the
     // level, at the price of one more dependent access per iteration. It pays
     // in a long pass, where warps have enough work to hide latency and
@@ -738,10 +770,10 @@ __device__ void process_items(const PeelArgs& a, ShT<kSample>& sh, const PassCtx
         }
       }
     }
+    if constexpr (kCombine) {
 #pragma unroll
-    for (int q = 0; q < kIlp; q++)
-      if (dq[q] > t) {
-        if constexpr (kCombine) {
+      for (int q = 0; q < kIlp; q++)
+        if (dq[q] > t) {
           // warp aggregation: the lanes of this slot that decrement the same
           // vertex send one atomic of their count; the lane whose interval
           // (old - cnt, old] holds k reports the crossing, so it is still
@@ -753,13 +785,23 @@ __device__ void process_items(const PeelArgs& a, ShT<kSample>& sh, const PassCtx
             const int old = atomicSub(a.deg + u[q], cnt);
             if (old > t && old - cnt <= t) cross |= 1u << q;
           }
-        } else {
-          ndec++;
-          const int old = atomicSub(a.deg + u[q], 1);
-          if (old == t + 1) cross |= 1u << q;
-          if (kWin && old == pc.win_hi) enter |= 1u << q;  // d~ drops into the level window
         }
+    } else {
+      // every decrement is issued before any result is used (dq then holds
+      // the values before)
+#pragma unroll
+      for (int q = 0; q < kIlp; q++) {
+        const bool dec = dq[q] > t;
+        ndec += dec ? 1 : 0;
+        dq[q] = INT_MIN;
+        if (dec) dq[q] = atomicSub(a.deg + u[q], 1);
       }
+#pragma unroll
+      for (int q = 0; q < kIlp; q++) {
+        if (dq[q] == t + 1) cross |= 1u << q;
+        if (kWin && dq[q] == pc.win_hi) enter |= 1u << q;  // d~ drops into the level window
+      }
+    }
     if (kWin && __any_sync(kFull, enter != 0)) {
       // append the vertices entering the window to the active list
 #pragma unroll
@@ -927,13 +969,10 @@ __device__ void hist_items(const PeelArgs& a, Shared& sh, const PassCtx& pc, uns
       u[q] = -1;
       if (base + q * kWarp < total) {
         const long long arc = mp.arc(base + q * kWarp, lane, before);
-        if (base + q * kWarp + lane < total) {
-          const int x = ld_stream_s32(a.adj + arc);
-          if ((unsigned)x < (unsigned)a.n) u[q] = x;
-          else raise_status(a, ST_NOT_SIMPLE);
-        }
+        if (base + q * kWarp + lane < total) u[q] = ld_stream_s32(a.adj + arc);
       }
     }
+    check_ids(a, u, total - base - lane);
     int dq[kIlp];
 #pragma unroll
     for (int q = 0; q < kIlp; q++) dq[q] = u[q] >= 0 ? __ldcg(a.deg + u[q]) : INT_MIN;
