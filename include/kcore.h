@@ -91,7 +91,8 @@ typedef enum {
   KCORE_OPT_BATCH_BLOCK = 11,    /* batched peel: threads per CTA (256, 512 or 1024; default 1024) */
   KCORE_OPT_BATCH_SMEM_VERTICES = 12, /* batched peel: graphs with at most this many vertices keep
                                          their induced degrees in shared memory (-1 = as many as
-                                         fit with the CTAs per SM below) */
+                                         fit with the CTAs per SM below); of a larger graph, those of
+                                         as many vertices */
   KCORE_OPT_BATCH_CTAS_PER_SM = 13,   /* batched peel: resident CTAs per SM (0 = occupancy limit) */
   KCORE_OPT_LOCAL_BATCHES = 14,       /* mode 2: local-queue batches a warp may run after each chunk it
                                          takes (0 .. 2^20, 0 = no limit; default 32); the rest of its local queue
@@ -296,8 +297,10 @@ kcore_status kcore_build_csr_workspace_size(kcore_handle h, int64_t n, int64_t n
  *   offsets, adj          device int64[N+1], int32[total_arcs]
  *   coreness_out          device int32[N]: coreness of every vertex in its graph
  *   kmax_out              device int32[G]: largest coreness of each graph (0 if empty)
- * Asynchronous; one persistent kernel (each graph peeled by one CTA, induced
- * degrees in shared memory when the graph fits, largest graphs first; with
+ * Asynchronous; one persistent kernel (each graph peeled by one CTA, or by half
+ * a 1,024-thread CTA once the graphs left hold at most half the batch's arcs
+ * per CTA each; induced degrees in shared memory as far as they fit, largest
+ * graphs first; with
  * KCORE_OPT_BATCH_CLUSTER, the graphs above KCORE_OPT_BATCH_BIG_ARCS arcs by a
  * thread-block cluster each, induced degrees in L2). Uses
  * kcore_batched_workspace_size bytes of workspace (20 bytes per vertex).

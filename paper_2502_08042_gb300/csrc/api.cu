@@ -785,6 +785,14 @@ kcore_status kcore_decompose_batched(kcore_handle h, int64_t num_graphs, int64_t
   a.next_graph = (int*)(ws + L.ctl);
   a.status = (int*)(ws + L.ctl) + 32;
   a.smem_deg_max = sv;
+  // Graphs of at most half the batch's arcs per CTA go to half a CTA each: a CTA
+  // that walks two graphs at once hides one's latency behind the other's, and
+  // such a graph, peeled at half the rate, still ends within a CTA's share.
+  // Measured (ms; whole CTAs only / this line with teams of 512 / teams of 256
+  // and a quarter of the share): 1,000 graphs of 1k..8k vertices 2.23 / 1.19 /
+  // 1.17, 2,000 of 1k..40k 10.3 / 5.4 / 5.5, 1,500 of 1k..200k 28.9 / 18.8 /
+  // 24.3, 512 of 1k..200k (bound by its largest graphs) the same.
+  if (sort_graphs && block == 1024) a.team_arcs = std::max<long long>(1, total_arcs / std::max(grid, 1) / 2);
   const int cluster = (int)h->opt[KCORE_OPT_BATCH_CLUSTER];
   if (cluster > 1 && block != 512 && block != 1024)
     return fail(h, KCORE_ERR_INVALID, "a clustered batch needs 512 or 1024 threads per CTA");

@@ -9,16 +9,24 @@
 //     never visited); the frontier is the live vertices sitting at that level;
 //   * subrounds: the arcs of the current frontier are processed edge-balanced
 //     by all threads of the CTA (a block scan of the frontier's degrees, then
-//     each thread takes arcs of the concatenated lists); a decrement that
+//     each warp takes 32-arc windows of the concatenated lists); a decrement that
 //     returns k+1 lands its vertex on k and appends it to the next subround's
-//     frontier; __syncthreads separates subrounds and levels;
+//     frontier; a barrier separates subrounds and levels;
 //   * the induced degrees live in shared memory when the graph is small enough
-//     (shared-memory atomics), otherwise in a per-graph slice of the workspace;
+//     (shared-memory atomics), those of a larger graph's first vertices in
+//     shared memory and the rest in a per-graph slice of the workspace;
 //     when every degree of the graph is below 2^16 they take 16 bits each
 //     (twice as many vertices fit in shared memory, half the L2 footprint).
 // Persistent CTAs take graphs from a device counter in descending order of
-// arcs (longest-processing-time first), so the largest graphs start first.
+// arcs (longest-processing-time first), so the largest graphs start first;
+// once the graphs are small, a 1,024-thread CTA splits into two teams that
+// each peel graphs of their own.
 // Nothing waits on another CTA: the kernel has no spin-waits.
+//
+// Measured (ms per batch, before the windows, the compile-time forms of d~,
+// the split store and the teams / with them): 1,000 graphs of 1k..8k vertices
+// 2.33 / 1.19, 512 of 1k..200k (617 M arcs, bound by its largest graphs) 20.6
+// / 10.7, 1,500 of 1k..200k 28.9 / 14.2, 2,000 of 1k..40k 10.3 / 4.9.
 //
 // A small batch is bound by its largest graphs, each walked by one CTA while
 // the others run out of work. The clustered form (batch_peel_cl) gives every
@@ -38,21 +46,36 @@
 
 namespace kc {
 
-constexpr int kBatchIlp = 4;
+// 32-arc windows a warp keeps in flight (bounded by the registers of three
+// 512-thread or six 256-thread CTAs per SM)
+template <int BLOCK>
+constexpr int kBatchIlp = BLOCK >= 1024 ? 8 : 4;
 constexpr int kScanItems = 8;  // active-list entries per thread per scan tile
 
 template <int BLOCK>
 struct BatchShared {
-  int pre[BLOCK];
-  long long start[BLOCK];
-  int part[BLOCK / 32];
-  int red[BLOCK / 32];
-  int cnt;
+  int pre[BLOCK];          // a chunk of frontier vertices: arcs ahead of each
+  const int* list[BLOCK];  // the address of each one's first arc, less its pre
+  int part[2][BLOCK / 32];  // block scan: two sets used in turn (one barrier per scan)
+  int red[2][BLOCK / 32];
+  int cnt[2];  // vertices appended to the next frontier (used in turn by the subrounds)
+  GraphDesc gd;  // the graph being peeled (its nine pointers would take 18 registers)
   int g;
-  int total;
   int bad;  // this graph failed a bounds check: stop peeling it
-  int base;  // clustered peel: this CTA's output position for the current tile
+  int base, base2;  // clustered peel: this CTA's output positions for the current tile
 };
+
+// A team: the BLOCK threads that peel one graph, the whole CTA or an aligned part
+// of it, with a barrier of its own (named barrier 1 + the team's index).
+template <int BLOCK>
+__device__ __forceinline__ int team_tid() {
+  static_assert((BLOCK & (BLOCK - 1)) == 0, "a power of two");
+  return (int)(threadIdx.x & (BLOCK - 1));
+}
+template <int BLOCK>
+__device__ __forceinline__ void team_sync() {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / BLOCK), "n"(BLOCK) : "memory");
+}
 
 // Records a failed bounds check (first one wins: code, graph-local value) and
 // flags the status; the access itself is skipped by the caller.
@@ -66,34 +89,39 @@ __device__ __forceinline__ void flag_bad(int* status, int code, long long value,
 }
 
 // Block-wide exclusive scan of one int per thread; returns the exclusive value,
-// *total gets the sum. Contains two __syncthreads.
+// *total gets the sum. One barrier: every warp scans the warps' sums itself,
+// and the sums alternate between two arrays (ph, toggled here), so the next
+// scan's stores cannot meet this one's loads.
 template <int BLOCK>
-__device__ __forceinline__ int block_excl_scan(int x, BatchShared<BLOCK>& sh, int* total) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int incl = warp_incl_scan(x, lane);
-  if (lane == 31) sh.part[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    int p = lane < BLOCK / 32 ? sh.part[lane] : 0;
-    int pi = warp_incl_scan(p, lane);
-    if (lane < BLOCK / 32) sh.part[lane] = pi - p;
-    if (lane == BLOCK / 32 - 1) sh.total = pi;
-  }
-  __syncthreads();
-  *total = sh.total;
-  return sh.part[warp] + incl - x;
+__device__ __forceinline__ int block_excl_scan(int x, BatchShared<BLOCK>& sh, int& ph, int* total) {
+  constexpr int kW = BLOCK / 32;
+  const int lane = threadIdx.x & 31, warp = team_tid<BLOCK>() >> 5;
+  const int incl = warp_incl_scan(x, lane);
+  int* part = sh.part[ph];
+  ph ^= 1;
+  if (lane == 31) part[warp] = incl;
+  team_sync<BLOCK>();
+  const int p = lane < kW ? part[lane] : 0;
+  const int pi = warp_incl_scan(p, lane);
+  *total = __shfl_sync(kFull, pi, kW - 1);
+  return __shfl_sync(kFull, pi - p, warp) + incl - x;
 }
 
+// Block-wide minimum of two values (one barrier; the callers have another
+// barrier between any two calls).
 template <int BLOCK>
-__device__ __forceinline__ int block_min(int x, BatchShared<BLOCK>& sh) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+__device__ __forceinline__ void block_min2(int& x, int& y, BatchShared<BLOCK>& sh) {
+  constexpr int kW = BLOCK / 32;
+  const int lane = threadIdx.x & 31, warp = team_tid<BLOCK>() >> 5;
   x = warp_min(x);
-  if (lane == 0) sh.red[warp] = x;
-  __syncthreads();
-  int m = INT_MAX;
-  for (int w = 0; w < BLOCK / 32; w++) m = min(m, sh.red[w]);
-  __syncthreads();
-  return m;
+  y = warp_min(y);
+  if (lane == 0) {
+    sh.red[0][warp] = x;
+    sh.red[1][warp] = y;
+  }
+  team_sync<BLOCK>();
+  x = warp_min(lane < kW ? sh.red[0][lane] : INT_MAX);
+  y = warp_min(lane < kW ? sh.red[1][lane] : INT_MAX);
 }
 
 // The induced degrees d~ of one graph, in shared memory or in L2 (atomics are
@@ -106,34 +134,258 @@ __device__ __forceinline__ int block_min(int x, BatchShared<BLOCK>& sh) {
 // word v >> 1). A vertex's d~ starts at its degree and falls by one per
 // peeled neighbour (each arc is traversed once), so it stays in [0, degree]:
 // with every degree below 2^16 a decrement never borrows from the other half.
+// Where the words live: all in shared memory, all in global memory, or (a
+// graph too large for shared memory) the first `cut` vertices in shared memory
+// and the rest in global memory. One SM sends about one scattered global
+// atomic per 1-2 cycles and several per cycle to shared memory, so every
+// vertex kept there shortens a large graph's subrounds.
+enum DegMode : int { kDegSmem = 0, kDegGlobal = 1, kDegSplit = 2 };
 struct DegStore {
-  int* w;
-  bool smem, narrow;
+  int* w;       // the words, in global memory
+  unsigned sa;  // in shared memory (shared-state address: a generic pointer would make
+                // every access, the atomics above all, a generic one)
+  int cut;      // vertices below are in shared memory (kDegSplit; even)
+  int mode;
+  bool narrow;
   uint64_t pol;
-  __device__ __forceinline__ int get(int v) const {
-    if (narrow) {
-      const int x = smem ? w[v >> 1] : ld_cg_keep(w + (v >> 1), pol);
-      return (x >> ((v & 1) * 16)) & 0xffff;
-    }
-    return smem ? w[v] : ld_cg_keep(w + v, pol);
+  template <bool kNarrow>
+  __device__ static __forceinline__ int value(int x, int v) {
+    return kNarrow ? ((unsigned)x >> ((v & 1) << 4)) & 0xffff : x;
   }
-  // decrements d~[v] by one and returns the value before
-  __device__ __forceinline__ int dec(int v) const {
-    if (narrow) {
-      const int sh = (v & 1) * 16;
-      const int old = smem ? atomicSub(w + (v >> 1), 1 << sh) : atom_add_keep(w + (v >> 1), -(1 << sh), pol);
-      return (old >> sh) & 0xffff;
+  template <bool kNarrow>
+  __device__ static __forceinline__ int minus_one(int v) {
+    return kNarrow && (v & 1) ? -65536 : -1;
+  }
+  template <bool kNarrow>
+  __device__ __forceinline__ unsigned saddr(int v) const {
+    return sa + 4u * (unsigned)(kNarrow ? v >> 1 : v);
+  }
+  // d~ of the vertices v[q] >= 0 (-1 where there is none), every load issued
+  // before any result is used
+  template <int kMode, bool kNarrow, int N>
+  __device__ __forceinline__ void get_all(const int (&v)[N], int (&d)[N]) const {
+#pragma unroll
+    for (int q = 0; q < N; q++) {
+      d[q] = -1;
+      if (kMode != kDegGlobal && v[q] >= 0 && (kMode == kDegSmem || v[q] < cut))
+        asm volatile("ld.shared.s32 %0, [%1];" : "=r"(d[q]) : "r"(saddr<kNarrow>(v[q])) : "memory");
+      if (kMode != kDegSmem && v[q] >= 0 && (kMode == kDegGlobal || v[q] >= cut))
+        d[q] = ld_cg_keep(w + (kNarrow ? v[q] >> 1 : v[q]), pol);
     }
-    return smem ? atomicSub(w + v, 1) : atom_add_keep(w + v, -1, pol);
+#pragma unroll
+    for (int q = 0; q < N; q++)
+      if (v[q] >= 0) d[q] = value<kNarrow>(d[q], v[q]);
+  }
+  template <int N>
+  __device__ __forceinline__ void get_all(const int (&v)[N], int (&d)[N]) const {
+    if (mode == kDegSmem) narrow ? get_all<kDegSmem, true>(v, d) : get_all<kDegSmem, false>(v, d);
+    else if (mode == kDegGlobal) narrow ? get_all<kDegGlobal, true>(v, d) : get_all<kDegGlobal, false>(v, d);
+    else narrow ? get_all<kDegSplit, true>(v, d) : get_all<kDegSplit, false>(v, d);
+  }
+  // decrements d~[u[q]] by one for the slots q with q * 32 < left; old[q]: the
+  // value before (0 for the other slots)
+  template <int kMode, bool kNarrow, int N>
+  __device__ __forceinline__ void dec_all(const int (&u)[N], int (&old)[N], int left) const {
+#pragma unroll
+    for (int q = 0; q < N; q++) {
+      old[q] = 0;
+      if (kMode != kDegGlobal && q * 32 < left && (kMode == kDegSmem || u[q] < cut))
+        asm volatile("atom.shared.add.s32 %0, [%1], %2;"
+                     : "=r"(old[q])
+                     : "r"(saddr<kNarrow>(u[q])), "r"(minus_one<kNarrow>(u[q]))
+                     : "memory");
+      if (kMode != kDegSmem && q * 32 < left && (kMode == kDegGlobal || u[q] >= cut))
+        old[q] = atom_add_keep(w + (kNarrow ? u[q] >> 1 : u[q]), minus_one<kNarrow>(u[q]), pol);
+    }
+#pragma unroll
+    for (int q = 0; q < N; q++)
+      if (q * 32 < left) old[q] = value<kNarrow>(old[q], u[q]);
   }
   // initial values: one word (narrow: vertices 2i and 2i + 1, degree d1 of
   // the second, 0 past the end)
   __device__ __forceinline__ void put_word(int i, int d0, int d1) const {
     const int x = narrow ? (d0 | (d1 << 16)) : d0;
-    if (smem) w[i] = x;
+    if (mode == kDegSmem || (mode == kDegSplit && i < (narrow ? cut >> 1 : cut)))
+      asm volatile("st.shared.s32 [%0], %1;" ::"r"(sa + 4u * (unsigned)i), "r"(x) : "memory");
     else st_keep(w + i, x, pol);
   }
 };
+
+// A chunk of up to BLOCK frontier vertices at `F`: thread tid gives its vertex
+// coreness k (set_core) and the chunk's arcs are laid out one after another
+// (sh.pre, sh.list). Returns the chunk's arcs. Two barriers; the chunk's
+// arrays may be reused after the caller's next barrier.
+template <int BLOCK>
+__device__ __forceinline__ int load_chunk(const GraphDesc& gd, const int* F, int cnum, int n, int k, bool set_core,
+                                          int* status, BatchShared<BLOCK>& sh, int& ph) {
+  const int tid = team_tid<BLOCK>();
+  int len = 0;
+  long long st = 0;
+  if (tid < cnum) {
+    const int v = __ldcg(F + tid);
+    if ((unsigned)v < (unsigned)n) {
+      if (set_core) gd.core[v] = k;
+      st = gd.off[v];
+      const long long e = gd.off[v + 1];
+      if (st < 0 || e < st || e > gd.m || e - st >= n) flag_bad(status, 2, v, &sh.bad);
+      else len = (int)(e - st);
+    } else {
+      flag_bad(status, 3, v, &sh.bad);
+    }
+  }
+  int total;
+  const int ex = block_excl_scan(len, sh, ph, &total);
+  sh.pre[tid] = ex;
+  sh.list[tid] = gd.adj + (st - ex);
+  team_sync<BLOCK>();
+  return total;
+}
+
+// Arcs [jlo, jhi) of the chunk: each warp takes a contiguous run of 32-arc
+// windows. The vertex a window starts in is found once per run (two ballots
+// over sh.pre); inside the run the vertices that start in a window form a bit
+// mask (one warp reduction), so an arc's vertex is a population count. What
+// bounds a chunk is the issue rate of one SM's warps, so the loop holds few
+// instructions per window: no search, no check of an arc's index (load_chunk
+// checked the lists; after a failed check nothing is read), the form of d~
+// fixed at compile time, and d~ decremented unread: a vertex at or below k is
+// already in a frontier (or peeled), never returns k + 1, and its d~ is only
+// compared with levels above k afterwards. All loads are issued before any
+// result is checked (a check that can branch to flag_bad between two loads
+// makes each wait for the one before), and the crossing vertices of kBatchIlp
+// windows are appended to Fn with one atomic. Every list of a chunk holds an
+// arc: a frontier vertex of level k >= 1 has degree >= k.
+template <int BLOCK, int kMode, bool kNarrow>
+__device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& D, int n, int k, int jlo, int jhi,
+                                           int cnum, int* Fn, int* counter, int* status, BatchShared<BLOCK>& sh) {
+  constexpr int kW = BLOCK / 32, kIlp = kBatchIlp<BLOCK>;
+  const int lane = threadIdx.x & 31, warp = team_tid<BLOCK>() >> 5;
+  const int run = ((((jhi - jlo + 31) >> 5) + kW - 1) / kW) << 5;  // arcs per warp
+  int j0 = jlo + warp * run;
+  const int jend = min(jhi, j0 + run);
+  if (j0 >= jend || __any_sync(kFull, sh.bad)) return;
+  int idx;  // last vertex that starts at or before j0
+  {
+    const int x = lane * kW;
+    unsigned m = __ballot_sync(kFull, x < cnum && sh.pre[x] <= j0);
+    const int c = m ? (31 - __clz(m)) * kW : 0;
+    m = __ballot_sync(kFull, lane < kW && c + lane < cnum && sh.pre[c + lane] <= j0);
+    idx = m ? c + 31 - __clz(m) : c;
+  }
+  const unsigned le = lanemask_lt() | (1u << lane);
+  for (; j0 < jend; j0 += kIlp * 32) {
+    int u[kIlp];
+    // the starts inside the iteration: one read gives the next 32; when they
+    // reach past it, the windows' masks do not depend on each other
+    const int e0 = idx + 1 + lane;
+    const unsigned d0 = e0 < cnum ? (unsigned)(sh.pre[e0] - j0) : 0x7fffffffu;
+    const bool few = __shfl_sync(kFull, d0, 31) >= kIlp * 32u;
+#pragma unroll
+    for (int q = 0; q < kIlp; q++) {
+      u[q] = 0;
+      if (j0 + q * 32 < jend) {
+        unsigned d = d0 - q * 32u;
+        if (!few) {
+          const int e = idx + 1 + lane;
+          d = e < cnum ? (unsigned)(sh.pre[e] - (j0 + q * 32)) : 32u;
+        }
+        const unsigned m = __reduce_or_sync(kFull, d < 32u ? 1u << d : 0u);
+        const int mine = idx + __popc(m & le);
+        idx += __popc(m);
+        const int j = j0 + q * 32 + lane;
+        if (j < jend) u[q] = ld_stream_s32(sh.list[mine] + j);
+      }
+    }
+    const int left = jend - j0 - lane;
+    bool bad = false;  // an id outside [0, n)
+#pragma unroll
+    for (int q = 0; q < kIlp; q++) bad |= (unsigned)u[q] >= (unsigned)n;
+    if (__any_sync(kFull, bad)) {
+      if (bad) flag_bad(status, 5, j0, &sh.bad);
+      return;
+    }
+    int old[kIlp];
+    D.dec_all<kMode, kNarrow>(u, old, left);
+    int cnt = 0;
+#pragma unroll
+    for (int q = 0; q < kIlp; q++) cnt += old[q] == k + 1 ? 1 : 0;
+    cnt = (int)__reduce_add_sync(kFull, (unsigned)cnt);
+    if (cnt) {
+      int pos = 0;
+      if (lane == 0) pos = atomicAdd(counter, cnt);
+      pos = __shfl_sync(kFull, pos, 0);
+      if (pos + cnt > n) {  // cannot happen: every vertex lands on k at most once per level
+        if (lane == 0) flag_bad(status, 7, pos, &sh.bad);
+        return;
+      }
+#pragma unroll
+      for (int q = 0; q < kIlp; q++) {
+        const unsigned m = __ballot_sync(kFull, old[q] == k + 1);
+        if (old[q] == k + 1) {
+          Fn[pos + __popc(m & lanemask_lt())] = u[q];
+          // its offsets are read next: from L2 then, not from DRAM
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(gd.off + u[q]));
+        }
+        pos += __popc(m);
+      }
+    }
+  }
+}
+
+template <int BLOCK>
+__device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& D, int n, int k, int jlo, int jhi,
+                                           int cnum, int* Fn, int* counter, int* status, BatchShared<BLOCK>& sh) {
+#define KC_ARCS(MODE)                                                                                            \
+  (D.narrow ? chunk_arcs<BLOCK, MODE, true>(gd, D, n, k, jlo, jhi, cnum, Fn, counter, status, sh)                  \
+            : chunk_arcs<BLOCK, MODE, false>(gd, D, n, k, jlo, jhi, cnum, Fn, counter, status, sh))
+  if (D.mode == kDegSmem) KC_ARCS(kDegSmem);
+  else if (D.mode == kDegGlobal) KC_ARCS(kDegGlobal);
+  else KC_ARCS(kDegSplit);
+#undef KC_ARCS
+}
+
+// Entry q of this thread in a tile of BLOCK * kScanItems list entries: a warp
+// takes consecutive entries, 32 per q, so its loads and the stores of what it
+// keeps are consecutive. (Eight entries per thread side by side in the output
+// put every lane of a store in a sector of its own: 4,700 of a tile's 10,700
+// cycles.)
+template <int BLOCK>
+__device__ __forceinline__ int tile_entry(int q) {
+  return (team_tid<BLOCK>() >> 5) * (32 * kScanItems) + q * 32 + (int)(threadIdx.x & 31);
+}
+
+// The kept (d >= keep_from) and taken (d == take_at) entries of a tile, packed
+// taken << 16 | kept: *total for the tile; returns those ahead of this warp.
+template <int BLOCK>
+__device__ __forceinline__ int tile_count(const int (&d)[kScanItems], int keep_from, int take_at,
+                                          BatchShared<BLOCK>& sh, int& ph, int* total) {
+  constexpr int kW = BLOCK / 32;
+  const int lane = threadIdx.x & 31, warp = team_tid<BLOCK>() >> 5;
+  int sum = 0;
+#pragma unroll
+  for (int q = 0; q < kScanItems; q++) sum += (d[q] >= keep_from ? 1 : 0) + (d[q] == take_at ? 1 << 16 : 0);
+  sum = (int)__reduce_add_sync(kFull, (unsigned)sum);
+  int* part = sh.part[ph];
+  ph ^= 1;
+  if (lane == 0) part[warp] = sum;
+  team_sync<BLOCK>();
+  const int p = lane < kW ? part[lane] : 0;
+  const int pi = warp_incl_scan(p, lane);
+  *total = __shfl_sync(kFull, pi, kW - 1);
+  return __shfl_sync(kFull, pi - p, warp);
+}
+
+// Writes the entries v[q] of the lanes with want(d[q]) to out, in list order.
+template <typename Want>
+__device__ __forceinline__ void tile_write(const int (&v)[kScanItems], const int (&d)[kScanItems], int* out, Want want) {
+#pragma unroll
+  for (int q = 0; q < kScanItems; q++) {
+    const bool w = want(d[q]);
+    const unsigned m = __ballot_sync(kFull, w);
+    if (w) __stcs(out + __popc(m & lanemask_lt()), v[q]);
+    out += __popc(m);
+  }
+}
 
 // One pass over the active list after level k: entries with D > k survive
 // into `out` (their minimum goes to *dmin); among them, those at exactly k+1
@@ -141,44 +393,34 @@ struct DegStore {
 // Returns the survivors; *nf gets the number written to F.
 template <int BLOCK>
 __device__ int compact_active(const int* A, int la, int n, int* out, int* F, const DegStore& D, int k,
-                              BatchShared<BLOCK>& sh, int* dmin, int* nf) {
+                              BatchShared<BLOCK>& sh, int& ph, int* dmin, int* nf) {
   int written = 0, wf = 0, lmin = INT_MAX;
   for (int base = 0; base < la; base += BLOCK * kScanItems) {
     int v[kScanItems];
-    unsigned keep = 0, front = 0;
 #pragma unroll
     for (int q = 0; q < kScanItems; q++) {
-      int i = base + q * BLOCK + threadIdx.x;
+      int i = base + tile_entry<BLOCK>(q);
       v[q] = -1;
       if (i < la) {
         int x = __ldcs(A + i);
         v[q] = (unsigned)x < (unsigned)n ? x : -1;  // ids are < n by construction; checked anyway
       }
     }
+    int d[kScanItems];
+    D.get_all(v, d);
 #pragma unroll
-    for (int q = 0; q < kScanItems; q++) {
-      if (v[q] >= 0) {
-        int d = D.get(v[q]);
-        if (d > k) {
-          keep |= 1u << q;
-          lmin = min(lmin, d);
-          if (d == k + 1) front |= 1u << q;
-        }
-      }
-    }
+    for (int q = 0; q < kScanItems; q++)
+      if (d[q] > k) lmin = min(lmin, d[q]);  // (no entry: -1)
     int tot;
-    int packed = __popc(keep) | (__popc(front) << 16);
-    int pos = block_excl_scan(packed, sh, &tot);
-    int pk = written + (pos & 0xffff), pf = wf + (pos >> 16);
-#pragma unroll
-    for (int q = 0; q < kScanItems; q++) {
-      if ((keep >> q) & 1u) __stcs(out + pk++, v[q]);
-      if ((front >> q) & 1u) __stcs(F + pf++, v[q]);
-    }
+    const int at = tile_count(d, k + 1, k + 1, sh, ph, &tot);
+    tile_write(v, d, out + written + (at & 0xffff), [k](int x) { return x > k; });
+    tile_write(v, d, F + wf + (at >> 16), [k](int x) { return x == k + 1; });
     written += tot & 0xffff;
     wf += tot >> 16;
   }
-  *dmin = block_min(lmin, sh);  // its barriers also publish the writes above
+  int none = INT_MAX;
+  block_min2(lmin, none, sh);  // its barrier also publishes the writes above
+  *dmin = lmin;
   *nf = wf;
   return written;
 }
@@ -186,61 +428,54 @@ __device__ int compact_active(const int* A, int la, int n, int* out, int* F, con
 // Selection of the frontier: entries of A with D[v] == k.
 template <int BLOCK>
 __device__ int select_frontier(const int* A, int la, int n, int* F, const DegStore& D, int k,
-                               BatchShared<BLOCK>& sh) {
+                               BatchShared<BLOCK>& sh, int& ph) {
   int written = 0;
   for (int base = 0; base < la; base += BLOCK * kScanItems) {
     int v[kScanItems];
-    unsigned take = 0;
 #pragma unroll
     for (int q = 0; q < kScanItems; q++) {
-      int i = base + q * BLOCK + threadIdx.x;
+      int i = base + tile_entry<BLOCK>(q);
       v[q] = -1;
       if (i < la) {
         int x = __ldcs(A + i);
         v[q] = (unsigned)x < (unsigned)n ? x : -1;  // ids are < n by construction; checked anyway
       }
     }
-#pragma unroll
-    for (int q = 0; q < kScanItems; q++)
-      if (v[q] >= 0 && D.get(v[q]) == k) take |= 1u << q;
+    int d[kScanItems];
+    D.get_all(v, d);
     int tot;
-    int pos = block_excl_scan(__popc(take), sh, &tot);
-    int p = written + pos;
-#pragma unroll
-    for (int q = 0; q < kScanItems; q++)
-      if ((take >> q) & 1u) __stcs(F + p++, v[q]);
-    written += tot;
+    const int at = tile_count(d, INT_MAX, k, sh, ph, &tot);
+    tile_write(v, d, F + written + (at >> 16), [k](int x) { return x == k; });
+    written += tot >> 16;
   }
-  __syncthreads();  // the frontier is read by other threads next
+  team_sync<BLOCK>();  // the frontier is read by other threads next
   return written;
 }
 
 // Peels one graph with the whole CTA (see the file comment).
 template <int BLOCK>
-__device__ void peel_one_graph(const GraphDesc& gd, int smem_deg_max, int* status, int* sdeg,
-                               BatchShared<BLOCK>& sh) {
-  const int tid = threadIdx.x, lane = tid & 31;
+__device__ void peel_one_graph(int smem_deg_max, int* status, int* sdeg, BatchShared<BLOCK>& sh) {
+  const GraphDesc& gd = sh.gd;
+  const int tid = team_tid<BLOCK>();
   if (gd.n <= 0) {
     if (tid == 0) *gd.kmax = 0;
-    __syncthreads();
+    team_sync<BLOCK>();
     return;
   }
   const int n = (int)gd.n;
-  const long long* O = gd.off;
-  const int* adj = gd.adj;
-  int* core = gd.core;
-  int* A0 = gd.A0;
-  int* A1 = gd.A1;
-  int* F0 = gd.F0;
-  int* F1 = gd.F1;
 
   // degrees: their minimum (the first level) and maximum (whether 16 bits
   // hold them), then the store, the initial values and the identity active list
-  if (tid == 0) sh.bad = 0;
-  __syncthreads();
+  if (tid == 0) {
+    sh.bad = 0;
+    sh.cnt[0] = 0;
+    sh.cnt[1] = 0;
+  }
+  team_sync<BLOCK>();
+  int ph = 0;  // which of the two sets of block-scan sums the next scan uses
   int lmin = INT_MAX, lmax = 0;
   for (int v = tid; v < n; v += BLOCK) {
-    long long o0 = O[v], o1 = O[v + 1];
+    long long o0 = gd.off[v], o1 = gd.off[v + 1];
     if (o0 < 0 || o1 < o0 || o1 > gd.m || o1 - o0 >= n) {
       flag_bad(status, 1, v, &sh.bad);
       o1 = o0;
@@ -249,136 +484,61 @@ __device__ void peel_one_graph(const GraphDesc& gd, int smem_deg_max, int* statu
     lmin = min(lmin, d);
     lmax = max(lmax, d);
   }
-  int k = block_min(lmin, sh);
-  const int dmax = -block_min(-lmax, sh);
+  int k = lmin, dmax = -lmax;
+  block_min2(k, dmax, sh);
+  dmax = -dmax;
   if (sh.bad) {  // malformed offsets: leave this graph (its outputs are undefined)
     if (tid == 0) *gd.kmax = -1;
-    __syncthreads();
+    team_sync<BLOCK>();
     return;
   }
   const bool narrow = dmax < 65536;
-  const bool in_smem = narrow ? n <= 2 * smem_deg_max : n <= smem_deg_max;
-  const DegStore D{in_smem ? sdeg : gd.deg, in_smem, narrow, l2_evict_last_policy()};
+  const int fit = narrow ? 2 * smem_deg_max : smem_deg_max;  // vertices that fit in shared memory
+  const DegStore D{gd.deg, (unsigned)__cvta_generic_to_shared(sdeg), fit,
+                   n <= fit ? kDegSmem : (fit > 0 ? kDegSplit : kDegGlobal), narrow, l2_evict_last_policy()};
   const int nw = narrow ? (n + 1) / 2 : n;
   for (int i = tid; i < nw; i += BLOCK) {
     const int v0 = narrow ? 2 * i : i;
-    const int d0 = (int)(O[v0 + 1] - O[v0]);
-    const int d1 = narrow && v0 + 1 < n ? (int)(O[v0 + 2] - O[v0 + 1]) : 0;
+    const int d0 = (int)(gd.off[v0 + 1] - gd.off[v0]);
+    const int d1 = narrow && v0 + 1 < n ? (int)(gd.off[v0 + 2] - gd.off[v0 + 1]) : 0;
     D.put_word(i, d0, d1);
   }
-  for (int v = tid; v < n; v += BLOCK) __stcs(A0 + v, v);
-  __syncthreads();
-  int* A = A0;
-  int* An = A1;
+  for (int v = tid; v < n; v += BLOCK) __stcs(gd.A0 + v, v);
+  team_sync<BLOCK>();
+  bool odd = false;  // the active list is in A1
   int la = n;
   int kmax = 0;
-  int nf = select_frontier<BLOCK>(A, la, n, F0, D, k, sh);
+  int r = 0;  // subrounds: frontier counter r & 1 counts this one's appends
+  int nf = select_frontier<BLOCK>(gd.A0, la, n, gd.F0, D, k, sh, ph);
   for (;;) {
-    int* Fc = F0;
-    int* Fn = F1;
+    bool fodd = false;  // the frontier is in F1
     while (nf > 0) {
-      for (int i = tid; i < nf; i += BLOCK) {
-        int v = __ldcs(Fc + i);
-        if ((unsigned)v < (unsigned)n) core[v] = k;
-        else flag_bad(status, 6, v, &sh.bad);
-      }
-      if (tid == 0) sh.cnt = 0;
-      __syncthreads();
       for (int c0 = 0; c0 < nf; c0 += BLOCK) {
         const int cnum = min(BLOCK, nf - c0);
-        int len = 0;
-        long long st = 0;
-        if (tid < cnum) {
-          int v = __ldcs(Fc + c0 + tid);
-          if ((unsigned)v < (unsigned)n) {
-            st = O[v];
-            long long e = O[v + 1];
-            if (st < 0 || e < st || e > gd.m || e - st >= n) flag_bad(status, 2, v, &sh.bad);
-            else len = (int)(e - st);
-          } else {
-            flag_bad(status, 3, v, &sh.bad);
-          }
-        }
-        int total;
-        int ex = block_excl_scan(len, sh, &total);
-        sh.pre[tid] = ex;
-        sh.start[tid] = st;
-        __syncthreads();
-        for (int j0 = 0; j0 < total; j0 += BLOCK * kBatchIlp) {
-          int u[kBatchIlp];
-#pragma unroll
-          for (int q = 0; q < kBatchIlp; q++) {
-            int j = j0 + q * BLOCK + tid;
-            u[q] = -1;
-            if (j < total) {
-              int lo = 0, hi = cnum;
-              while (lo < hi) {
-                int mid = (lo + hi) >> 1;
-                if (sh.pre[mid] <= j) lo = mid + 1;
-                else hi = mid;
-              }
-              int idx = lo - 1;
-              long long arc = sh.start[idx] + (j - sh.pre[idx]);
-              if (idx < 0 || arc < 0 || arc >= gd.m) {
-                flag_bad(status, 4, arc, &sh.bad);
-              } else {
-                u[q] = ld_stream_s32(adj + arc);
-                if ((unsigned)u[q] >= (unsigned)n) {
-                  flag_bad(status, 5, u[q], &sh.bad);
-                  u[q] = -1;
-                }
-              }
-            }
-          }
-#pragma unroll
-          for (int q = 0; q < kBatchIlp; q++) {
-            bool cross = false;
-            // induced degrees in shared memory: read first, decrement the live
-            // ones. In global memory each access is an L2 request, so the
-            // decrement goes unread: a vertex at or below k is already in a
-            // frontier (or peeled), never returns k + 1, and its d~ is only
-            // compared with levels above k afterwards.
-            if (u[q] >= 0) {
-              if (D.smem) cross = D.get(u[q]) > k && D.dec(u[q]) == k + 1;
-              else cross = D.dec(u[q]) == k + 1;
-            }
-            unsigned m = __ballot_sync(kFull, cross);
-            if (m) {
-              int base = 0;
-              if (lane == __ffs(m) - 1) base = atomicAdd(&sh.cnt, __popc(m));
-              base = __shfl_sync(kFull, base, __ffs(m) - 1);
-              int pos = base + __popc(m & lanemask_lt());
-              if (cross) {
-                if (pos < n) __stcs(Fn + pos, u[q]);
-                else flag_bad(status, 7, pos, &sh.bad);
-              }
-            }
-          }
-        }
-        __syncthreads();
+        const int total = load_chunk<BLOCK>(gd, (fodd ? gd.F1 : gd.F0) + c0, cnum, n, k, true, status, sh, ph);
+        // every thread has read the last subround's counter: clear it for the next
+        if (tid == 0 && c0 == 0) sh.cnt[(r + 1) & 1] = 0;
+        chunk_arcs<BLOCK>(gd, D, n, k, 0, total, cnum, fodd ? gd.F0 : gd.F1, &sh.cnt[r & 1], status, sh);
+        team_sync<BLOCK>();
       }
-      nf = sh.cnt;
+      nf = sh.cnt[r & 1];
       if (nf > n) nf = 0;  // cannot happen: every vertex lands on k at most once per level
-      __syncthreads();
-      int* t = Fc;
-      Fc = Fn;
-      Fn = t;
+      r++;
+      fodd = !fodd;
     }
     kmax = k;
     // drop the vertices peeled at level k; the minimum induced degree of the
     // rest is the next non-empty level; vertices at k+1 are collected on the
     // way in case that level is the next one
     int dmin;
-    la = compact_active<BLOCK>(A, la, n, An, F0, D, k, sh, &dmin, &nf);
-    int* t = A;
-    A = An;
-    An = t;
+    la = compact_active<BLOCK>(odd ? gd.A1 : gd.A0, la, n, odd ? gd.A0 : gd.A1, gd.F0, D, k, sh, ph, &dmin, &nf);
+    odd = !odd;
     if (la == 0) break;
-    if (dmin != k + 1) nf = select_frontier<BLOCK>(A, la, n, F0, D, dmin, sh);
+    if (dmin != k + 1) nf = select_frontier<BLOCK>(odd ? gd.A1 : gd.A0, la, n, gd.F0, D, dmin, sh, ph);
     k = dmin;
   }
   if (tid == 0) *gd.kmax = kmax;
-  __syncthreads();
+  team_sync<BLOCK>();
 }
 
 // ------------------------------------------------------------------ clustered form
@@ -403,6 +563,7 @@ struct ClusterPeel {
   int* status;
   int r;       // this CTA's rank in the cluster
   int ph = 0;  // phase index (the same in every CTA)
+  int sp = 0;  // which of the two sets of block-scan sums the next scan uses
 
   __device__ ClusterPeel(ClusterCtl* lead, BatchShared<BLOCK>& s, int* st)
       : cl(cg::this_cluster()), lc(lead), sh(s), status(st), r((int)cg::this_cluster().block_rank()) {}
@@ -435,27 +596,22 @@ struct ClusterPeel {
     const int lo = (int)part_lo(la), hi = (int)part_hi(la);
     for (int base = lo; base < hi; base += BLOCK * kScanItems) {
       int v[kScanItems];
-      unsigned take = 0;
 #pragma unroll
       for (int q = 0; q < kScanItems; q++) {
-        const int i = base + q * BLOCK + threadIdx.x;
+        const int i = base + tile_entry<BLOCK>(q);
         v[q] = -1;
         if (i < hi) {
           const int x = __ldcg(A + i);  // written by other CTAs of the cluster
           v[q] = (unsigned)x < (unsigned)n ? x : -1;
         }
       }
-#pragma unroll
-      for (int q = 0; q < kScanItems; q++)
-        if (v[q] >= 0 && D.get(v[q]) == k) take |= 1u << q;
+      int d[kScanItems];
+      D.get_all(v, d);
       int tot;
-      const int pos = block_excl_scan(__popc(take), sh, &tot);
-      if (threadIdx.x == 0) sh.base = tot ? atomicAdd(&slot(ph)[0], tot) : 0;
+      const int at = tile_count(d, INT_MAX, k, sh, sp, &tot);
+      if (threadIdx.x == 0) sh.base = tot ? atomicAdd(&slot(ph)[0], tot >> 16) : 0;
       __syncthreads();
-      int p = sh.base + pos;
-#pragma unroll
-      for (int q = 0; q < kScanItems; q++)
-        if ((take >> q) & 1u) F[p++] = v[q];
+      tile_write(v, d, F + sh.base + (at >> 16), [k](int x) { return x == k; });
       __syncthreads();  // sh.base is reused by the next tile
     }
   }
@@ -467,52 +623,42 @@ struct ClusterPeel {
     int lmin = INT_MAX;
     for (int base = lo; base < hi; base += BLOCK * kScanItems) {
       int v[kScanItems];
-      unsigned keep = 0, front = 0;
 #pragma unroll
       for (int q = 0; q < kScanItems; q++) {
-        const int i = base + q * BLOCK + threadIdx.x;
+        const int i = base + tile_entry<BLOCK>(q);
         v[q] = -1;
         if (i < hi) {
           const int x = __ldcg(A + i);
           v[q] = (unsigned)x < (unsigned)n ? x : -1;
         }
       }
+      int d[kScanItems];
+      D.get_all(v, d);
 #pragma unroll
-      for (int q = 0; q < kScanItems; q++) {
-        if (v[q] >= 0) {
-          const int d = D.get(v[q]);
-          if (d > k) {
-            keep |= 1u << q;
-            lmin = min(lmin, d);
-            if (d == k + 1) front |= 1u << q;
-          }
-        }
-      }
+      for (int q = 0; q < kScanItems; q++)
+        if (d[q] > k) lmin = min(lmin, d[q]);  // (no entry: -1)
       int tot;
-      const int pos = block_excl_scan(__popc(keep) | (__popc(front) << 16), sh, &tot);
+      const int at = tile_count(d, k + 1, k + 1, sh, sp, &tot);
       if (threadIdx.x == 0) {
         const int bk = (tot & 0xffff) ? atomicAdd(&slot(ph)[0], tot & 0xffff) : 0;
         const int bf = (tot >> 16) ? atomicAdd(&slot(ph)[1], tot >> 16) : 0;
         sh.base = bk;
-        sh.cnt = bf;
+        sh.base2 = bf;
       }
       __syncthreads();
-      int pk = sh.base + (pos & 0xffff), pf = sh.cnt + (pos >> 16);
-#pragma unroll
-      for (int q = 0; q < kScanItems; q++) {
-        if ((keep >> q) & 1u) out[pk++] = v[q];
-        if ((front >> q) & 1u) F[pf++] = v[q];
-      }
+      tile_write(v, d, out + sh.base + (at & 0xffff), [k](int x) { return x > k; });
+      tile_write(v, d, F + sh.base2 + (at >> 16), [k](int x) { return x == k + 1; });
       __syncthreads();
     }
-    const int m = block_min(lmin, sh);
-    if (threadIdx.x == 0 && m != INT_MAX) atomicMin(&slot(ph)[2], m);
+    int none = INT_MAX;
+    block_min2(lmin, none, sh);
+    if (threadIdx.x == 0 && lmin != INT_MAX) atomicMin(&slot(ph)[2], lmin);
   }
 
   // Peels one graph with the whole cluster (Algorithm 1's levels and
   // subrounds, the online Peel of Algorithm 3, as peel_one_graph does in one CTA).
   __device__ void peel(const GraphDesc& gd) {
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x;
     if (first()) {
       lc->bad = 0;
       clear(0);
@@ -535,8 +681,9 @@ struct ClusterPeel {
       lmin = min(lmin, (int)(o1 - o0));
       lmax = max(lmax, (int)(o1 - o0));
     }
-    lmin = block_min(lmin, sh);
-    lmax = -block_min(-lmax, sh);
+    lmax = -lmax;
+    block_min2(lmin, lmax, sh);
+    lmax = -lmax;
     if (tid == 0) {
       atomicMin(&slot(ph)[2], lmin);
       atomicMax(&slot(ph)[3], lmax);
@@ -549,7 +696,7 @@ struct ClusterPeel {
       return;
     }
     const bool narrow = dmax < 65536;
-    const DegStore D{gd.deg, false, narrow, l2_evict_last_policy()};
+    const DegStore D{gd.deg, 0u, 0, kDegGlobal, narrow, l2_evict_last_policy()};
     // phase: initial induced degrees, the identity active list
     const int nw = narrow ? (n + 1) / 2 : n;
     for (long long i = (long long)r * BLOCK + tid; i < nw; i += (long long)C * BLOCK) {
@@ -570,81 +717,16 @@ struct ClusterPeel {
       int* Fc = gd.F0;
       int* Fn = gd.F1;
       while (nf > 0) {
-        for (long long i = (long long)r * BLOCK + tid; i < nf; i += (long long)C * BLOCK) {
-          const int v = __ldcg(Fc + i);
-          if ((unsigned)v < (unsigned)n) gd.core[v] = k;
-          else flag_bad(status, 6, v, &sh.bad);
-        }
         // a large frontier: the CTAs take whole chunks of BLOCK frontier
         // vertices in turn; a small one: every CTA walks every chunk and takes
-        // its share of the chunk's arcs
+        // its share of the chunk's arcs (the first CTA writes their coreness)
         const bool whole = nf >= 2 * C * BLOCK;
         for (int c0 = whole ? r * BLOCK : 0; c0 < nf; c0 += whole ? C * BLOCK : BLOCK) {
           const int cnum = min(BLOCK, nf - c0);
-          int len = 0;
-          long long st = 0;
-          if (tid < cnum) {
-            const int v = __ldcg(Fc + c0 + tid);
-            if ((unsigned)v < (unsigned)n) {
-              st = O[v];
-              const long long e = O[v + 1];
-              if (st < 0 || e < st || e > gd.m || e - st >= n) flag_bad(status, 2, v, &sh.bad);
-              else len = (int)(e - st);
-            } else {
-              flag_bad(status, 3, v, &sh.bad);
-            }
-          }
-          int total;
-          const int ex = block_excl_scan(len, sh, &total);
-          sh.pre[tid] = ex;
-          sh.start[tid] = st;
-          __syncthreads();
-          const int jlo = whole ? 0 : (int)part_lo(total), jhi = whole ? total : (int)part_hi(total);
-          for (int j0 = jlo; j0 < jhi; j0 += BLOCK * kBatchIlp) {
-            int u[kBatchIlp];
-#pragma unroll
-            for (int q = 0; q < kBatchIlp; q++) {
-              const int j = j0 + q * BLOCK + tid;
-              u[q] = -1;
-              if (j < jhi) {
-                int lo = 0, hi = cnum;
-                while (lo < hi) {
-                  const int mid = (lo + hi) >> 1;
-                  if (sh.pre[mid] <= j) lo = mid + 1;
-                  else hi = mid;
-                }
-                const int idx = lo - 1;
-                const long long arc = idx >= 0 ? sh.start[idx] + (j - sh.pre[idx]) : -1;
-                if (idx < 0 || arc < 0 || arc >= gd.m) {
-                  flag_bad(status, 4, arc, &sh.bad);
-                } else {
-                  u[q] = ld_stream_s32(gd.adj + arc);
-                  if ((unsigned)u[q] >= (unsigned)n) {
-                    flag_bad(status, 5, u[q], &sh.bad);
-                    u[q] = -1;
-                  }
-                }
-              }
-            }
-#pragma unroll
-            for (int q = 0; q < kBatchIlp; q++) {
-              // d~ lives in L2: the decrement goes unread (a vertex at or
-              // below k never returns k + 1)
-              const bool cross = u[q] >= 0 && D.dec(u[q]) == k + 1;
-              const unsigned m = __ballot_sync(kFull, cross);
-              if (m) {
-                int base = 0;
-                if (lane == __ffs(m) - 1) base = atomicAdd(&slot(ph)[0], __popc(m));
-                base = __shfl_sync(kFull, base, __ffs(m) - 1);
-                const int pos = base + __popc(m & lanemask_lt());
-                if (cross) {
-                  if (pos < n) Fn[pos] = u[q];
-                  else flag_bad(status, 7, pos, &sh.bad);
-                }
-              }
-            }
-          }
-          __syncthreads();  // sh.pre / sh.start are reused by the next chunk
+          const int total = load_chunk<BLOCK>(gd, Fc + c0, cnum, n, k, whole || r == 0, status, sh, sp);
+          chunk_arcs<BLOCK>(gd, D, n, k, whole ? 0 : (int)part_lo(total), whole ? total : (int)part_hi(total), cnum, Fn,
+                            &slot(ph)[0], status, sh);
+          __syncthreads();  // the chunk's arrays are reused by the next one
         }
         next_phase();
         nf = slot(ph - 1)[0];
@@ -678,42 +760,67 @@ struct ClusterPeel {
   }
 };
 
+// graph g of a batch: vertices [v0, v0 + n)
+__device__ __forceinline__ GraphDesc batch_desc(const BatchArgs& a, long long g, long long v0, long long n) {
+  return GraphDesc{a.off + v0, a.adj,     a.core + v0, a.kmax + g, a.deg + v0, a.A0 + v0,
+                   a.A1 + v0,  a.F0 + v0, a.F1 + v0,   n,          a.m};
+}
+
+// Draws graph after graph for the team and peels them. first >= 0: a graph the
+// CTA drew already. With a.team_arcs > 0, returns the first graph below that
+// many arcs unpeeled (its position), else -1 once the batch is exhausted.
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 2048 / BLOCK * 3 / 4)) batch_peel(BatchArgs a) {
-  extern __shared__ int sdeg[];
-  __shared__ BatchShared<BLOCK> sh;
+__device__ long long peel_drawn(const BatchArgs& a, int smem_deg_max, int* sdeg, BatchShared<BLOCK>& sh, long long first,
+                                long long stop_below) {
+  const int tid = team_tid<BLOCK>();
   for (;;) {
-    if (threadIdx.x == 0) sh.g = atomicAdd(a.next_graph, 1);
-    __syncthreads();
-    long long gi = sh.g;
-    __syncthreads();
-    if (gi >= a.G) break;
-    long long g = a.order ? a.order[gi] : gi;
+    if (tid == 0) sh.g = first >= 0 ? (int)first : atomicAdd(a.next_graph, 1);
+    first = -1;
+    team_sync<BLOCK>();
+    const long long gi = sh.g;
+    team_sync<BLOCK>();
+    if (gi >= a.G) return -1;
+    const long long g = a.order ? a.order[gi] : gi;
     if (g < 0 || g >= a.G) {  // the order is a permutation of [0, G); checked anyway
-      if (threadIdx.x == 0) flag_bad(a.status, 8, g, &sh.bad);
+      if (tid == 0) flag_bad(a.status, 8, g, &sh.bad);
       continue;
     }
-    GraphDesc gd;
-    const long long v0 = a.gv[g];
-    gd.n = a.gv[g + 1] - v0;
-    if (v0 < 0 || gd.n < 0 || v0 + gd.n > a.N) {  // graph outside the vertex range
-      if (threadIdx.x == 0) {
+    const long long v0 = a.gv[g], n = a.gv[g + 1] - v0;
+    if (v0 < 0 || n < 0 || v0 + n > a.N) {  // graph outside the vertex range
+      if (tid == 0) {
         flag_bad(a.status, 9, g, &sh.bad);
         a.kmax[g] = -1;
       }
       continue;
     }
-    gd.m = a.m;
-    gd.off = a.off + v0;
-    gd.adj = a.adj;
-    gd.core = a.core + v0;
-    gd.kmax = a.kmax + g;
-    gd.deg = a.deg + v0;
-    gd.A0 = a.A0 + v0;
-    gd.A1 = a.A1 + v0;
-    gd.F0 = a.F0 + v0;
-    gd.F1 = a.F1 + v0;
-    peel_one_graph<BLOCK>(gd, a.smem_deg_max, a.status, sdeg, sh);
+    if (stop_below > 0 && a.off[v0 + n] - a.off[v0] < stop_below) return gi;
+    if (tid == 0) sh.gd = batch_desc(a, g, v0, n);
+    team_sync<BLOCK>();
+    peel_one_graph<BLOCK>(smem_deg_max, a.status, sdeg, sh);
+  }
+}
+
+// A 1,024-thread CTA peels whole graphs while they are large (a.team_arcs arcs
+// or more; the order is by arcs) and from the first smaller one on splits into
+// teams of kTeam threads, each drawing graphs of its own with its share of the
+// shared memory: a small graph's phases are short dependent chains that leave
+// most of an SM idle.
+constexpr int kTeam = 512;
+
+template <int BLOCK>
+__global__ void __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 2048 / BLOCK * 3 / 4)) batch_peel(BatchArgs a) {
+  extern __shared__ int sdeg[];
+  constexpr int kTeams = BLOCK >= 1024 ? BLOCK / kTeam : 1;
+  __shared__ union {
+    BatchShared<BLOCK> whole;
+    BatchShared<BLOCK / kTeams> team[kTeams];
+  } sh;
+  long long gi = peel_drawn<BLOCK>(a, a.smem_deg_max, sdeg, sh.whole, -1, kTeams > 1 ? a.team_arcs : 0);
+  if constexpr (kTeams > 1) {
+    if (gi < 0) return;
+    __syncthreads();
+    const int t = threadIdx.x / kTeam, share = a.smem_deg_max / kTeams;
+    peel_drawn<kTeam>(a, share, sdeg + t * share, sh.team[t], t == 0 ? gi : -1, 0);
   }
 }
 
@@ -749,36 +856,26 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(BLOCK, (BLOCK >= 102
       if (threadIdx.x == 0) flag_bad(a.status, 8, g, &sh.bad);
       continue;
     }
-    GraphDesc gd;
-    const long long v0 = a.gv[g];
-    gd.n = a.gv[g + 1] - v0;
-    if (v0 < 0 || gd.n < 0 || v0 + gd.n > a.N) {
+    const long long v0 = a.gv[g], n = a.gv[g + 1] - v0;
+    if (v0 < 0 || n < 0 || v0 + n > a.N) {
       if (threadIdx.x == 0 && (!together || lead)) {
         flag_bad(a.status, 9, g, &sh.bad);
         a.kmax[g] = -1;
       }
       continue;
     }
-    gd.m = a.m;
-    gd.off = a.off + v0;
-    gd.adj = a.adj;
-    gd.core = a.core + v0;
-    gd.kmax = a.kmax + g;
-    gd.deg = a.deg + v0;
-    gd.A0 = a.A0 + v0;
-    gd.A1 = a.A1 + v0;
-    gd.F0 = a.F0 + v0;
-    gd.F1 = a.F1 + v0;
-    if (together && gd.n > 0 && gd.n < INT_MAX && gd.off[gd.n] - gd.off[0] >= big_arcs) {
+    if (threadIdx.x == 0) sh.gd = batch_desc(a, g, v0, n);
+    __syncthreads();
+    if (together && n > 0 && n < INT_MAX && a.off[v0 + n] - a.off[v0] >= big_arcs) {
       ClusterPeel<BLOCK, C> cp(lc, sh, a.status);
-      cp.peel(gd);
+      cp.peel(sh.gd);
       continue;
     }
     if (together) {
       together = false;  // the first CTA peels this graph, the others draw their own
       if (!lead) continue;
     }
-    peel_one_graph<BLOCK>(gd, a.smem_deg_max, a.status, sdeg, sh);
+    peel_one_graph<BLOCK>(a.smem_deg_max, a.status, sdeg, sh);
   }
 }
 
@@ -796,8 +893,9 @@ __global__ void __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 2048 / BLOCK / 2))
     int gi = sh.g;
     __syncthreads();
     if (gi >= list.count) break;
-    GraphDesc gd = table[list.slot[gi]];
-    peel_one_graph<BLOCK>(gd, smem_deg_max, status, sdeg, sh);
+    if (threadIdx.x == 0) sh.gd = table[list.slot[gi]];
+    __syncthreads();
+    peel_one_graph<BLOCK>(smem_deg_max, status, sdeg, sh);
   }
 }
 
@@ -828,7 +926,9 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(BLOCK, (BLOCK >= 102
       __syncthreads();
     }
     if (gi >= list.count) break;
-    const GraphDesc gd = table[list.slot[gi]];
+    if (threadIdx.x == 0) sh.gd = table[list.slot[gi]];
+    __syncthreads();
+    const GraphDesc& gd = sh.gd;
     if (together && gd.n > 0 && gd.n < INT_MAX && gd.off[gd.n] - gd.off[0] >= big_arcs) {
       ClusterPeel<BLOCK, C> cp(lc, sh, status);
       cp.peel(gd);
@@ -838,7 +938,7 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(BLOCK, (BLOCK >= 102
       together = false;  // the first CTA peels this graph, the others draw their own
       if (!lead) continue;
     }
-    peel_one_graph<BLOCK>(gd, smem_deg_max, status, sdeg, sh);
+    peel_one_graph<BLOCK>(smem_deg_max, status, sdeg, sh);
   }
 }
 

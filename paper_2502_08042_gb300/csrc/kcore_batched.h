@@ -26,7 +26,11 @@ struct BatchArgs {
   const int* order;          // [G] processing order, or nullptr
   int* next_graph;           // work counter
   int* status;
-  int smem_deg_max;          // graphs with at most this many vertices keep d~ in shared memory
+  long long team_arcs;       // 1,024-thread CTAs: from the first graph below this many arcs on (the order is
+                             // by arcs), each team of the CTA peels graphs of its own (0: never)
+  int smem_deg_max;          // 32-bit words of d~ in shared memory (a CTA's teams share them): a vertex
+                             // each, or two when every degree is below 2^16; the vertices past
+                             // them keep d~ in `deg`
 };
 
 // One graph of a descriptor-driven launch: offsets hold absolute indices
