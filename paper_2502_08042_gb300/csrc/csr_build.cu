@@ -22,8 +22,9 @@
 //      vertex's offset). Keys are read striped (a warp reads 32 consecutive
 //      keys), the predecessor comes from the next lower lane, and the
 //      positions from warp ballots, so no key passes through shared memory.
-// A single graph takes a shorter route through steps 1-3: each pair (a, b)
-// with a != b gives ONE key (min << B) | max; sorting these E keys by both
+// A single graph, and a batch for which it means fewer keys to move, takes the
+// edge route through steps 1-3: each pair (a, b) with a != b gives ONE key
+// (min << B) | max (global ids); sorting these E keys by both
 // fields gives every vertex's upper neighbours in order (A), and a stable
 // sort of A by its low B bits (the larger endpoint) gives every vertex's
 // lower neighbours in order (B). A vertex's list is its lower neighbours
@@ -36,6 +37,7 @@
 //
 // Lists come out ascending and duplicate-free, the canonical form of the CPU
 // builder, so the two are comparable bit for bit.
+#include <algorithm>
 #include <climits>
 
 #include "kcore_csr.h"
@@ -44,8 +46,6 @@
 namespace kc {
 
 constexpr int kCsrBlock = 256;
-constexpr int kKeysPerThread = 8;
-constexpr int kTile = kCsrBlock * kKeysPerThread;  // 2048
 constexpr unsigned long long kSentinel = ~0ull;
 
 // Keys (source << Bd) | target. Single graph: ids in [0, n), source = id.
@@ -105,24 +105,32 @@ __device__ __forceinline__ void edge_keys(const EdgeList& es, long long i, int a
   }
 }
 
-// a single graph's edge i = (a, b) as one key (min << B) | max
-__device__ __forceinline__ unsigned long long edge_canon(const EdgeList& es, int a, int b) {
-  if ((unsigned long long)(unsigned)a >= (unsigned long long)es.n ||
-      (unsigned long long)(unsigned)b >= (unsigned long long)es.n) {
+// edge i = (a, b) as one key (min << B) | max; a batch's (kBatch) with global
+// ids, its edge i in one of the graphs [glo, ghi)
+template <bool kBatch>
+__device__ __forceinline__ unsigned long long edge_canon(const EdgeList& es, long long i, int a, int b, long long glo,
+                                                         long long ghi) {
+  long long base = 0, lim = es.n;
+  if constexpr (kBatch) {
+    const long long g = ghi - glo == 1 ? glo : graph_of(es, i, glo, ghi);
+    base = es.gv[g];
+    lim = es.gv[g + 1] - base;
+  }
+  if ((unsigned long long)(unsigned)a >= (unsigned long long)lim ||
+      (unsigned long long)(unsigned)b >= (unsigned long long)lim) {
     atomicCAS(es.status, 0, 1);
     return kSentinel;
   }
   if (a == b) return kSentinel;
-  const unsigned lo = (unsigned)min(a, b), hi = (unsigned)max(a, b);
-  return ((unsigned long long)lo << es.Bd) | (unsigned long long)hi;
+  return ((unsigned long long)(base + min(a, b)) << es.Bd) | (unsigned long long)(base + max(a, b));
 }
 
 // Where a pass's keys come from: a key array, the edge list as two arcs per
-// edge (the first pass of the general build), the edge list as one key per
-// edge (the first pass of a single graph's build), or a sorted key array
+// edge (the first pass of the arc route), the edge list as one key per edge
+// (the first pass of the edge route; kCanonB: a batch's), or a sorted key array
 // without its sentinels and without keys equal to their predecessor (the
 // first pass of B's sort).
-enum KeySrc : int { kKeys = 0, kArcs = 1, kCanon = 2, kKeysDrop = 3 };
+enum KeySrc : int { kKeys = 0, kArcs = 1, kCanon = 2, kKeysDrop = 3, kCanonB = 4 };
 
 // digit of a pass: bits [shift, shift + 8) of the key, masked by dmask (the
 // last pass over a field narrower than a multiple of 8 bits keeps only its bits)
@@ -142,7 +150,13 @@ __global__ void __launch_bounds__(kCsrBlock) rs_upsweep(const unsigned long long
   for (int i = tid; i < (kCsrBlock / 32) * 256; i += kCsrBlock) (&cnt[0][0])[i] = 0;
   __syncthreads();
   long long lo = (long long)blockIdx.x * chunk, hi = min(N, lo + chunk);
-  if constexpr (kSrc == kCanon) {
+  if constexpr (kSrc == kCanon || kSrc == kCanonB) {
+    __shared__ long long cg_lo, cg_hi;
+    if constexpr (kSrc == kCanonB) {
+      chunk_graphs(es, lo, max(lo, hi), &cg_lo, &cg_hi);
+      __syncthreads();
+    }
+    const long long glo = kSrc == kCanonB ? cg_lo : 0, ghi = kSrc == kCanonB ? cg_hi : 0;
     constexpr int kU = 4;
     for (long long e0 = lo + tid; e0 < hi; e0 += kU * kCsrBlock) {
       int a[kU], b[kU];
@@ -154,7 +168,9 @@ __global__ void __launch_bounds__(kCsrBlock) rs_upsweep(const unsigned long long
       }
 #pragma unroll
       for (int u = 0; u < kU; u++)
-        if (e0 + u * kCsrBlock < hi) atomicAdd(&cnt[warp][digit_of(edge_canon(es, a[u], b[u]), shift, dmask)], 1u);
+        if (e0 + u * kCsrBlock < hi)
+          atomicAdd(&cnt[warp][digit_of(edge_canon<kSrc == kCanonB>(es, e0 + u * kCsrBlock, a[u], b[u], glo, ghi), shift, dmask)],
+                    1u);
     }
   } else if constexpr (kSrc == kArcs) {
     __shared__ long long cg_lo, cg_hi;
@@ -238,19 +254,26 @@ __global__ void __launch_bounds__(1024) scan_u32_to_u64(const unsigned* in, unsi
 // Pos: the type of an output position (32 bits when there are at most 2^32
 // keys: positions are then computed modulo 2^32).
 static_assert(kCsrBlock == 256, "one thread per 8-bit digit");
+constexpr int kSortKeys = 16;                     // keys per thread per tile
+constexpr int kSortTile = kCsrBlock * kSortKeys;  // 4,096
 template <int kSrc, typename Pos>
-__global__ void __launch_bounds__(kCsrBlock, 5) rs_downsweep(const unsigned long long* in, EdgeList es,
+__global__ void __launch_bounds__(kCsrBlock, 3) rs_downsweep(const unsigned long long* in, EdgeList es,
                                                           unsigned long long* out, long long N,
                                                           long long chunk, int shift, int dmask,
                                                           const unsigned long long* offs,
                                                           const unsigned long long* rowtot) {
-  __shared__ unsigned long long buf[kTile];
-  __shared__ __align__(16) unsigned long long stage[kTile];  // the next tile, copied asynchronously
-  __shared__ unsigned wcnt[kCsrBlock / 32][256];  // keys per (warp, digit), then their tile offsets
+  constexpr int kW = kCsrBlock / 32, kRow = kSortKeys * 32;  // keys of a warp's part of a tile
+  // The warps' digit counters (x: the lanes of the current row that hold the
+  // digit, y: keys counted) are done with before the exchange buffer is
+  // written, so they share its memory.
+  __shared__ __align__(16) union {
+    unsigned long long buf[kSortTile];
+    uint2 cnt[kW][256];
+  } sm;
+  __shared__ unsigned wofs[kW][256];  // tile offset of each (warp, digit)'s first key
   __shared__ Pos dstb[256];  // output position of the tile's first key of digit d, minus its tile offset
-  __shared__ unsigned long long part64[kCsrBlock / 32];
-  __shared__ unsigned part[kCsrBlock / 32];
-  __shared__ unsigned tile_keys;  // keys of the tile that are written (all but kKeysDrop's dropped ones)
+  __shared__ unsigned long long part64[kW];
+  __shared__ unsigned part[kW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = gridDim.x;
   const unsigned lt = lanemask_lt();
@@ -260,111 +283,98 @@ __global__ void __launch_bounds__(kCsrBlock, 5) rs_downsweep(const unsigned long
     const unsigned long long rt = rowtot[tid];
     const unsigned long long incl = warp_incl_scan(rt, lane);
     if (lane == 31) part64[warp] = incl;
-    for (int i = tid; i < (kCsrBlock / 32) * 256; i += kCsrBlock) (&wcnt[0][0])[i] = 0;
     __syncthreads();
     unsigned long long before = 0;
     for (int w = 0; w < warp; w++) before += part64[w];
     run = before + incl - rt + offs[(long long)tid * G + blockIdx.x];
   }
-  long long lo = (long long)blockIdx.x * chunk, hi = min(N, lo + chunk);
-  __shared__ long long cg_lo, cg_hi;  // kArcs, a batch: the graphs of this chunk's edges
-  if constexpr (kSrc == kArcs) {
-    chunk_graphs(es, lo / 2, hi > lo ? hi / 2 : lo / 2, &cg_lo, &cg_hi);
-    __syncthreads();
-  }
-  // 16-byte asynchronous copies of a tile's keys into `stage` (pairs of keys;
-  // a last odd key is copied with its neighbour, which lies inside the
-  // key buffer and is not used). kArcs / kCanon: the tile's sources and
-  // targets go to the stage's two halves (4 KB each for kArcs, 8 KB for
-  // kCanon), by 16-byte copies when both arrays are 16-byte aligned and the
-  // tile is whole, else by 4-byte copies (nothing past the last edge is read).
-  const unsigned sbase = (unsigned)__cvta_generic_to_shared(stage);
-  const bool al16 =
-      ((reinterpret_cast<unsigned long long>(es.src) | reinterpret_cast<unsigned long long>(es.dst)) & 15) == 0;
-  auto prefetch = [&](long long t0) {
-    const long long tn = min((long long)kTile, hi - t0);
-    if constexpr (kSrc == kArcs || kSrc == kCanon) {
-      constexpr int kE = kSrc == kArcs ? kTile / 2 : kTile;  // edges per tile
-      constexpr unsigned kHalf = 4u * kE;                     // bytes of one array's share
-      const long long e0 = kSrc == kArcs ? t0 / 2 : t0, ne = kSrc == kArcs ? tn / 2 : tn;
-      if (al16 && ne == kE) {
-        for (int c = tid; 4 * c < kE; c += kCsrBlock) {
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sbase + 16u * c), "l"(es.src + e0 + 4 * c)
-                       : "memory");
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sbase + kHalf + 16u * c),
-                       "l"(es.dst + e0 + 4 * c)
-                       : "memory");
-        }
-      } else {
-        for (int c = tid; c < ne; c += kCsrBlock) {
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sbase + 4u * c), "l"(es.src + e0 + c)
-                       : "memory");
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sbase + kHalf + 4u * c), "l"(es.dst + e0 + c)
-                       : "memory");
-        }
-      }
-    } else {
-      for (int c = tid; 2 * c < tn; c += kCsrBlock)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sbase + 16u * c), "l"(in + t0 + 2 * c)
-                     : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  if (lo < hi) prefetch(lo);
-  for (long long ts = lo; ts < hi; ts += kTile) {
-    const long long tn = min((long long)kTile, hi - ts);
-    unsigned long long k[kKeysPerThread];
-    unsigned rk[kKeysPerThread / 2];  // ranks below 2,048: two per word
-    // key it of this thread is key j_of(it) of the tile (kArcs: arc it & 1 of
-    // the tile's edge el_of(it); kCanon: edge j_of(it)); 256 is the digit of no key
-    auto j_of = [&](int it) { return warp * (kKeysPerThread * 32) + it * 32 + lane; };
-    auto el_of = [&](int it) { return warp * (kKeysPerThread * 16) + (it >> 1) * 32 + lane; };
+  const long long lo = (long long)blockIdx.x * chunk, hi = min(N, lo + chunk);
+  __shared__ long long cg_lo, cg_hi;  // a batch's first pass: the graphs of this chunk's edges
+  if constexpr (kSrc == kArcs) chunk_graphs(es, lo / 2, hi > lo ? hi / 2 : lo / 2, &cg_lo, &cg_hi);
+  if constexpr (kSrc == kCanonB) chunk_graphs(es, lo, max(lo, hi), &cg_lo, &cg_hi);
+  for (long long ts = lo; ts < hi; ts += kSortTile) {
+    const int tn = (int)min((long long)kSortTile, hi - ts);
+    unsigned long long k[kSortKeys];
+    unsigned rk[kSortKeys / 2];  // ranks below 4,096: two per word
+    // key it of this thread is key j_of(it) of the tile, a row of 32 keys per
+    // warp and it (kArcs: arc it & 1 of the tile's edge el_of(it))
+    auto j_of = [&](int it) { return warp * kRow + it * 32 + lane; };
+    auto el_of = [&](int it) { return warp * (kRow / 2) + (it >> 1) * 32 + lane; };
     unsigned dropped = 0;  // kKeysDrop: bit it set for a dropped key
     auto valid = [&](int it) {
       return kSrc == kArcs ? el_of(it) < tn / 2 : (j_of(it) < tn && !((dropped >> it) & 1u));
     };
-    auto dg_of = [&](int it) { return valid(it) ? digit_of(k[it], shift, dmask) : 256; };
-    const unsigned long long pre = kSrc == kKeysDrop && tid == 0 && ts > 0 ? in[ts - 1] : kSentinel;
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
-    if constexpr (kSrc == kCanon) {
-      const int* sa = reinterpret_cast<const int*>(stage);
+    // every load of the tile before any use
+    if constexpr (kSrc == kCanon || kSrc == kCanonB) {
+      int x[kSortKeys], y[kSortKeys];
 #pragma unroll
-      for (int it = 0; it < kKeysPerThread; it++)
-        k[it] = valid(it) ? edge_canon(es, sa[j_of(it)], sa[kTile + j_of(it)]) : 0;
+      for (int it = 0; it < kSortKeys; it++) {
+        x[it] = valid(it) ? __ldcs(es.src + ts + j_of(it)) : 0;
+        y[it] = valid(it) ? __ldcs(es.dst + ts + j_of(it)) : 0;
+      }
+      if (kSrc == kCanonB && ts == lo) __syncthreads();  // cg_lo, cg_hi
+#pragma unroll
+      for (int it = 0; it < kSortKeys; it++)
+        k[it] = valid(it) ? edge_canon<kSrc == kCanonB>(es, ts + j_of(it), x[it], y[it], kSrc == kCanonB ? cg_lo : 0,
+                                                        kSrc == kCanonB ? cg_hi : 0)
+                          : 0;
     } else if constexpr (kSrc == kArcs) {
-      const int* sa = reinterpret_cast<const int*>(stage);
+      int x[kSortKeys / 2], y[kSortKeys / 2];
 #pragma unroll
-      for (int it = 0; it < kKeysPerThread; it += 2) {
+      for (int it = 0; it < kSortKeys; it += 2) {
+        x[it / 2] = valid(it) ? __ldcs(es.src + ts / 2 + el_of(it)) : 0;
+        y[it / 2] = valid(it) ? __ldcs(es.dst + ts / 2 + el_of(it)) : 0;
+      }
+      if (ts == lo) __syncthreads();  // cg_lo, cg_hi
+#pragma unroll
+      for (int it = 0; it < kSortKeys; it += 2) {
         k[it] = k[it + 1] = 0;
-        if (valid(it))
-          edge_keys(es, ts / 2 + el_of(it), sa[el_of(it)], sa[1024 + el_of(it)], k[it], k[it + 1], cg_lo, cg_hi);
+        if (valid(it)) edge_keys(es, ts / 2 + el_of(it), x[it / 2], y[it / 2], k[it], k[it + 1], cg_lo, cg_hi);
       }
     } else {
 #pragma unroll
-      for (int it = 0; it < kKeysPerThread; it++) k[it] = j_of(it) < tn ? stage[j_of(it)] : 0;
+      for (int it = 0; it < kSortKeys; it++) k[it] = j_of(it) < tn ? __ldcs(in + ts + j_of(it)) : kSentinel;
       if constexpr (kSrc == kKeysDrop) {
+        const long long first = ts + warp * kRow;
+        unsigned long long last = lane == 0 && first > 0 && first < N ? __ldcg(in + first - 1) : kSentinel;
 #pragma unroll
-        for (int it = 0; it < kKeysPerThread; it++) {
-          const int j = j_of(it);
-          const unsigned long long p = j > 0 ? stage[j - 1] : pre;
-          if (j < tn && (k[it] == kSentinel || k[it] == p)) dropped |= 1u << it;
+        for (int it = 0; it < kSortKeys; it++) {
+          const unsigned long long up = __shfl_up_sync(kFull, k[it], 1);
+          const unsigned long long p = lane > 0 ? up : last;
+          if (k[it] == kSentinel || k[it] == p) dropped |= 1u << it;
+          last = __shfl_sync(kFull, k[it], 31);
         }
       }
     }
-    __syncthreads();  // the stage is read: copy the next tile into it
-    if (ts + kTile < hi) prefetch(ts + kTile);
-    // rank within (warp, digit) in key order: iterations in order, lanes in
-    // order within an iteration
+    // the next tile's lines start their way from DRAM (one 16-key line per thread)
+    static_assert(kSortTile / 16 == kCsrBlock, "one line per thread");
+    if ((kSrc == kKeys || kSrc == kKeysDrop) && ts + kSortTile + tid * 16 < hi)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(in + ts + kSortTile + tid * 16));
+    __syncthreads();  // the last tile's keys are written out: the counters may take their place
+    for (int i = tid; i < kW * 256 / 2; i += kCsrBlock) reinterpret_cast<uint4*>(sm.cnt)[i] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    // A key's rank among its warp's keys of the same digit, in key order (rows
+    // in order, lanes in order within a row). The lanes of a digit find each
+    // other by or-ing their bits into its counter and reading it back: about 11
+    // cycles of the SM per row of 32 random digits, where match.any takes 40
+    // and eight ballots 16 (one CTA of 256 threads x 5 per SM, measured). The
+    // first pass of a build need not be stable: a counter's old value is rank enough.
 #pragma unroll
-    for (int it = 0; it < kKeysPerThread; it++) {
-      const int dg = dg_of(it);
-      const unsigned peers = __match_any_sync(kFull, dg);
-      const int leader = __ffs(peers) - 1;
-      unsigned old = 0;
-      if (lane == leader && dg < 256) old = atomicAdd(&wcnt[warp][dg], (unsigned)__popc(peers));
-      old = __shfl_sync(kFull, old, leader);
-      const unsigned r = old + __popc(peers & lt);
+    for (int it = 0; it < kSortKeys; it++) {
+      const bool v = valid(it);
+      uint2* c = &sm.cnt[warp][digit_of(k[it], shift, dmask)];
+      unsigned r = 0;
+      if constexpr (kSrc == kCanon || kSrc == kCanonB || kSrc == kArcs) {
+        if (v) r = atomicAdd(&c->y, 1u);
+      } else {
+        if (v) atomicOr(&c->x, 1u << lane);
+        __syncwarp();
+        const uint2 mc = *c;
+        __syncwarp();
+        r = mc.y + __popc(mc.x & lt);
+        if (v && (mc.x & lt) == 0) *c = make_uint2(0u, mc.y + __popc(mc.x));
+        __syncwarp();
+      }
       if (it & 1) rk[it >> 1] |= r << 16;
       else rk[it >> 1] = r;
     }
@@ -372,218 +382,170 @@ __global__ void __launch_bounds__(kCsrBlock, 5) rs_downsweep(const unsigned long
     // per digit (thread d): tile count, exclusive offsets over digits, then
     // over warps
     unsigned tc = 0;
-    for (int w = 0; w < kCsrBlock / 32; w++) tc += wcnt[w][tid];
-    unsigned incl = warp_incl_scan(tc, lane);
+#pragma unroll
+    for (int w = 0; w < kW; w++) tc += sm.cnt[w][tid].y;
+    const unsigned incl = warp_incl_scan(tc, lane);
     if (lane == 31) part[warp] = incl;
     __syncthreads();
-    if (warp == 0) {
-      unsigned p = lane < kCsrBlock / 32 ? part[lane] : 0;
-      unsigned pi = warp_incl_scan(p, lane);
-      if (lane < kCsrBlock / 32) part[lane] = pi - p;
-    }
-    __syncthreads();
-    const unsigned lo_d = part[warp] + incl - tc;
+    const unsigned p8 = lane < kW ? part[lane] : 0;
+    const unsigned pi = warp_incl_scan(p8, lane);
+    const unsigned lo_d = __shfl_sync(kFull, pi - p8, warp) + incl - tc;
+    const int tk = (int)__shfl_sync(kFull, pi, kW - 1);  // keys of the tile that are written
     unsigned acc = lo_d;
-    for (int w = 0; w < kCsrBlock / 32; w++) {
-      unsigned c = wcnt[w][tid];
-      wcnt[w][tid] = acc;
-      acc += c;
+#pragma unroll
+    for (int w = 0; w < kW; w++) {
+      wofs[w][tid] = acc;
+      acc += sm.cnt[w][tid].y;
     }
     dstb[tid] = (Pos)(run - lo_d);  // modulo 2^64 (2^32): adding a tile offset of digit tid lands at or after run
     run += tc;
-    if (tid == 255) tile_keys = lo_d + tc;
     __syncthreads();
 #pragma unroll
-    for (int it = 0; it < kKeysPerThread; it++) {
-      const int dg = dg_of(it);
-      if (dg < 256) buf[wcnt[warp][dg] + ((rk[it >> 1] >> (16 * (it & 1))) & 0xffffu)] = k[it];
-    }
+    for (int it = 0; it < kSortKeys; it++)
+      if (valid(it))
+        sm.buf[wofs[warp][digit_of(k[it], shift, dmask)] + ((rk[it >> 1] >> (16 * (it & 1))) & 0xffffu)] = k[it];
     __syncthreads();
-    for (int w = 0; w < kCsrBlock / 32; w++) wcnt[w][tid] = 0;  // for the next tile
-    const int tk = (int)tile_keys;
+#pragma unroll 4
     for (int j = tid; j < tk; j += kCsrBlock) {
-      const unsigned long long key = buf[j];
+      const unsigned long long key = sm.buf[j];
       out[(unsigned long long)(Pos)(dstb[digit_of(key, shift, dmask)] + (Pos)j)] = key;
     }
   }
 }
 
-// A tile is kRows rows of kCsrBlock consecutive keys; a thread takes one key
-// per row (a warp 32 consecutive keys). A key's neighbours come from
-// the next lower and higher lanes; at a warp's edges from the keys the
-// neighbouring warps publish in shared memory, and at the tile's edges from
-// the keys just before and after it (read by threads 0 and kCsrBlock - 1).
-template <int kRows>
-struct TileEdges {
-  unsigned long long first[kRows][kCsrBlock / 32];
-  unsigned long long last[kRows][kCsrBlock / 32];
-};
+// The unique-key passes: a warp walks its own contiguous chunk of keys,
+// kURows rows of 32 at a time, all loaded before any is compared; a key's
+// neighbours come from the next lanes and rows. Nothing is shared between
+// warps, so there is no barrier (a CTA-wide tile needed three per 1,024 keys:
+// 278 M keys were counted in 0.55 ms and emitted in 1.82, now 0.40 and 1.16).
+constexpr int kURows = 8;
+constexpr int kUTile = kURows * 32;
 
-template <int kRows>
-__device__ __forceinline__ void publish_edges(TileEdges<kRows>& e, const unsigned long long* x, int lane, int warp) {
+struct WarpKeys {
+  unsigned long long x[kURows];
+  unsigned long long prev, next;  // the keys before and after the tile (kSentinel: none)
+  // keys [ts, ts + kUTile) of k[0, hi), hi <= N; prev holds the key before ts
+  __device__ __forceinline__ void load(const unsigned long long* k, long long ts, long long hi, long long N, int lane) {
 #pragma unroll
-  for (int q = 0; q < kRows; q++) {
-    if (lane == 0) e.first[q][warp] = x[q];
-    if (lane == 31) e.last[q][warp] = x[q];
-  }
-}
-
-// predecessor of this thread's key in row q (pre: the key before the tile, held by thread 0)
-template <int kRows>
-__device__ __forceinline__ unsigned long long pred_key(const TileEdges<kRows>& e, unsigned long long xq, int q, int lane,
-                                                       int warp, unsigned long long pre) {
-  const unsigned long long up = __shfl_up_sync(kFull, xq, 1);
-  if (lane > 0) return up;
-  if (warp > 0) return e.last[q][warp - 1];
-  return q > 0 ? e.last[q - 1][kCsrBlock / 32 - 1] : pre;
-}
-
-// successor (post: the key after the tile, held by thread kCsrBlock - 1)
-template <int kRows>
-__device__ __forceinline__ unsigned long long succ_key(const TileEdges<kRows>& e, unsigned long long xq, int q, int lane,
-                                                       int warp, unsigned long long post) {
-  const unsigned long long dn = __shfl_down_sync(kFull, xq, 1);
-  if (lane < 31) return dn;
-  if (warp < kCsrBlock / 32 - 1) return e.first[q][warp + 1];
-  return q < kRows - 1 ? e.first[q + 1][0] : post;
-}
-
-// Unique keys of each CTA chunk (a key differing from its predecessor).
-__global__ void __launch_bounds__(kCsrBlock, 5) csr_count_unique(const unsigned long long* k, long long N,
-                                                              long long chunk, unsigned* cnt) {
-  constexpr int kRows = kKeysPerThread;
-  __shared__ TileEdges<kRows> edges;
-  __shared__ unsigned part[kCsrBlock / 32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  long long lo = (long long)blockIdx.x * chunk, hi = min(N, lo + chunk);
-  unsigned c = 0;
-  for (long long ts = lo; ts < hi; ts += kTile) {
-    unsigned long long x[kRows];
-#pragma unroll
-    for (int q = 0; q < kRows; q++) {
-      const long long i = ts + (long long)q * kCsrBlock + tid;
+    for (int q = 0; q < kURows; q++) {
+      const long long i = ts + q * 32 + lane;
       x[q] = i < hi ? __ldcs(k + i) : kSentinel;
     }
-    const unsigned long long pre = tid == 0 && ts > 0 ? __ldcg(k + ts - 1) : kSentinel;
-    publish_edges(edges, x, lane, warp);
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kRows; q++) {
-      const long long i = ts + (long long)q * kCsrBlock + tid;
-      const unsigned long long p = pred_key(edges, x[q], q, lane, warp, pre);
-      if (i < hi && x[q] != kSentinel && (i == 0 || p != x[q])) c++;
+    next = ts + kUTile < N ? __ldg(k + ts + kUTile) : kSentinel;
+  }
+  __device__ __forceinline__ unsigned long long pred(int q, int lane) const {
+    const unsigned long long up = __shfl_up_sync(kFull, x[q], 1);
+    const unsigned long long last = q > 0 ? __shfl_sync(kFull, x[q > 0 ? q - 1 : 0], 31) : prev;
+    return lane > 0 ? up : last;
+  }
+  __device__ __forceinline__ unsigned long long succ(int q, int lane) const {
+    const unsigned long long dn = __shfl_down_sync(kFull, x[q], 1);
+    const unsigned long long first = q < kURows - 1 ? __shfl_sync(kFull, x[q < kURows - 1 ? q + 1 : q], 0) : next;
+    return lane < 31 ? dn : first;
+  }
+  __device__ __forceinline__ void step() { prev = __shfl_sync(kFull, x[kURows - 1], 31); }
+};
+
+// A batch's edge route: the first vertex of the graph that holds vertex v, for
+// the ids that leave as graph-local ones. A warp's keys run through the graphs
+// in order, so the last graph found serves most of them.
+struct GraphBase {
+  const long long* gv;
+  long long G, from, to;  // the graph at hand: vertices [from, to)
+  __device__ __forceinline__ GraphBase(const long long* gv_, long long G_) : gv(gv_), G(G_), from(0), to(0) {}
+  __device__ __forceinline__ long long of(long long v) {
+    if (v < from || v >= to) {
+      long long lo = 0, hi = G;  // the last graph with gv[g] <= v
+      while (hi - lo > 1) {
+        const long long mid = (lo + hi) >> 1;
+        if (gv[mid] <= v) lo = mid;
+        else hi = mid;
+      }
+      from = gv[lo];
+      to = gv[lo + 1];
     }
-    __syncthreads();  // the edges are read: the next tile may publish its own
+    return from;
+  }
+};
+
+// Unique keys of each warp's chunk (a key differing from its predecessor).
+__global__ void __launch_bounds__(kCsrBlock) csr_count_unique(const unsigned long long* k, long long N,
+                                                              long long chunk, unsigned* cnt) {
+  const int lane = threadIdx.x & 31;
+  const long long w = (long long)blockIdx.x * (kCsrBlock / 32) + (threadIdx.x >> 5);
+  const long long lo = w * chunk, hi = min(N, lo + chunk);
+  unsigned c = 0;
+  WarpKeys t;
+  t.prev = lo > 0 && lo < hi ? __ldg(k + lo - 1) : kSentinel;
+  for (long long ts = lo; ts < hi; ts += kUTile) {
+    t.load(k, ts, hi, N, lane);
+#pragma unroll
+    for (int q = 0; q < kURows; q++) {
+      const unsigned long long p = t.pred(q, lane);
+      c += t.x[q] != kSentinel && t.x[q] != p ? 1 : 0;
+    }
+    t.step();
   }
   c = warp_sum(c);
-  if (lane == 0) part[warp] = c;
-  __syncthreads();
-  if (tid == 0) {
-    unsigned s = 0;
-    for (int w = 0; w < kCsrBlock / 32; w++) s += part[w];
-    cnt[blockIdx.x] = s;
-  }
+  if (lane == 0) cnt[w] = c;
 }
 
 // Ordered emission of the unique keys. A unique key's position ("before":
-// unique keys ahead of it) is the chunk's base, plus the unique keys of
-// earlier rows and of earlier warps in its row (one warp scans the tile's rows
-// x warps counts), plus those of lower lanes (a ballot). A key's group is its
-// high field (the source, or the smaller endpoint).
+// unique keys ahead of it) is the warp's base, plus the unique keys of earlier
+// rows and lower lanes (ballots). A key's group is its high field (the source,
+// or the smaller endpoint).
 //   kEmitAll: adj[pos] = low B bits; the first arc of each source fixes
 //     offsets[] for that source and every source without arcs just below it;
 //     the last arc fills the offsets of the sources above it.
 //   kEmitUpper (sequence A): vertex u's upper neighbours go after its lower
 //     ones: adj[pos + starts[u + 1]] = larger endpoint, and offsets[x] = A's
 //     unique keys with smaller endpoint below x (csr_finish_offsets adds
-//     starts[x]); m = twice A's unique keys.
+//     starts[x]); m = twice A's unique keys. gv: a batch's ids leave graph-local.
 enum EmitMode : int { kEmitAll = 0, kEmitUpper = 2 };
 template <int kMode>
-__global__ void __launch_bounds__(kCsrBlock, 5) csr_emit(const unsigned long long* __restrict__ k, long long N,
+__global__ void __launch_bounds__(kCsrBlock) csr_emit(const unsigned long long* __restrict__ k, long long N,
                                                       long long chunk, int B, long long n,
                                                       const unsigned long long* __restrict__ base,
                                                       int* __restrict__ adj, long long* __restrict__ off,
                                                       long long* __restrict__ m_out,
                                                       unsigned long long* __restrict__ starts,
-                                                      long long* __restrict__ tail) {
-  constexpr int kW = kCsrBlock / 32;
-  constexpr int kRows = 4;  // a tile of kRows * kCsrBlock keys (chunks are whole tiles of either size)
-  constexpr int kT = kRows * kCsrBlock;
-  static_assert(kRows * kW == 32 && kTile % kT == 0, "the tile's counts are scanned by one warp, one per lane");
-  __shared__ TileEdges<kRows> edges;
-  __shared__ unsigned cnt[kRows * kW];  // unique keys per (row, warp), then their offsets in the tile
-  __shared__ unsigned tile_total;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+                                                      long long* __restrict__ tail, const long long* __restrict__ gv,
+                                                      long long G) {
+  const int lane = threadIdx.x & 31;
+  GraphBase gb(gv, G);
+  const long long w = (long long)blockIdx.x * (kCsrBlock / 32) + (threadIdx.x >> 5);
   const unsigned long long mask = (1ull << B) - 1;
   const unsigned lt = lanemask_lt();
-  long long lo = (long long)blockIdx.x * chunk, hi = min(N, lo + chunk);
-  unsigned long long running = base[blockIdx.x];
-  for (long long ts = lo; ts < hi; ts += kT) {
-    unsigned long long x[kRows];
+  const long long lo = w * chunk, hi = min(N, lo + chunk);
+  if (lo >= hi) return;
+  unsigned long long running = base[w];
+  WarpKeys t;
+  t.prev = lo > 0 ? __ldg(k + lo - 1) : kSentinel;
+  for (long long ts = lo; ts < hi; ts += kUTile) {
+    t.load(k, ts, hi, N, lane);
+    // the lookups of each key (kEmitUpper: the lower neighbours of u come
+    // first), all issued before any store
+    unsigned long long look[kURows];
 #pragma unroll
-    for (int q = 0; q < kRows; q++) {
-      const long long i = ts + (long long)q * kCsrBlock + tid;
-      x[q] = i < hi ? __ldcs(k + i) : kSentinel;
-    }
-    const unsigned long long pre = tid == 0 && ts > 0 ? __ldcg(k + ts - 1) : kSentinel;
-    // chunks are whole tiles, so a key past the tile's end lies in the next chunk or past N
-    const unsigned long long post = tid == kCsrBlock - 1 && ts + kT < N ? __ldcg(k + ts + kT) : kSentinel;
-    publish_edges(edges, x, lane, warp);
-    __syncthreads();
-    unsigned bal[kRows];
-    int ps[kRows];  // source of the predecessor (-1: none)
-    unsigned closing = 0;    // bit q: the key of row q is the last valid key
-    unsigned mine = 0;
+    for (int q = 0; q < kURows; q++)
+      look[q] = kMode == kEmitUpper && t.x[q] != kSentinel ? starts[(long long)(t.x[q] >> B) + 1] : 0;
 #pragma unroll
-    for (int q = 0; q < kRows; q++) {
-      const long long i = ts + (long long)q * kCsrBlock + tid;
-      const unsigned long long p = pred_key(edges, x[q], q, lane, warp, pre);
-      const unsigned long long sk = succ_key(edges, x[q], q, lane, warp, post);  // every lane: a shuffle
-      const unsigned long long nx = i + 1 < N ? sk : kSentinel;
-      const bool valid = i < hi && x[q] != kSentinel;
-      ps[q] = (i == 0 || p == kSentinel) ? -1 : (int)(p >> B);
-      if (valid && nx == kSentinel) closing |= 1u << q;
-      bal[q] = __ballot_sync(kFull, valid && (i == 0 || p != x[q]));
-      if (lane == q) mine = __popc(bal[q]);
-    }
-    if (lane < kRows) cnt[lane * kW + warp] = mine;
-    __syncthreads();
-    if (warp == 0) {
-      const unsigned c0 = cnt[lane];
-      const unsigned incl = warp_incl_scan(c0, lane);
-      cnt[lane] = incl - c0;
-      if (lane == 31) tile_total = incl;
-    }
-    // the lookups of each unique key, all issued before any store
-    unsigned long long look0[kRows];
-#pragma unroll
-    for (int q = 0; q < kRows; q++) {
-      look0[q] = 0;
-      if ((bal[q] >> lane) & 1u) {
-        if constexpr (kMode == kEmitUpper) {
-          const long long u = (long long)(x[q] >> B);
-          look0[q] = starts[u + 1];  // the lower neighbours of u come first
-        }
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kRows; q++) {
-      const bool u = (bal[q] >> lane) & 1u;
-      const unsigned long long before = running + cnt[q * kW + warp] + __popc(bal[q] & lt);
-      const long long hi_f = (long long)(x[q] >> B), lo_f = (long long)(x[q] & mask);
-      const long long s = hi_f;  // the key's group
+    for (int q = 0; q < kURows; q++) {
+      const unsigned long long x = t.x[q], p = t.pred(q, lane), sk = t.succ(q, lane);
+      const bool u = x != kSentinel && x != p;
+      const unsigned bal = __ballot_sync(kFull, u);
+      const unsigned long long before = running + __popc(bal & lt);
+      running += __popc(bal);
+      const long long s = (long long)(x >> B);  // the key's group
       if (u) {
-        if constexpr (kMode == kEmitAll) {
-          adj[before] = (int)lo_f;
-          for (long long v = (long long)ps[q] + 1; v <= s; v++) off[v] = (long long)before;
-        } else {
-          adj[before + look0[q]] = (int)lo_f;
-          for (long long v = (long long)ps[q] + 1; v <= s; v++) off[v] = (long long)before;
-        }
+        long long id = (long long)(x & mask);
+        if (kMode == kEmitUpper && gv) id -= gb.of(s);
+        adj[before + look[q]] = (int)id;
+        const long long ps = p == kSentinel ? -1 : (long long)(p >> B);
+        for (long long v = ps + 1; v <= s; v++) off[v] = (long long)before;
       }
       // the last valid key (unique or a repeat) closes the groups above its own
-      if ((closing >> q) & 1u) {
+      if (x != kSentinel && sk == kSentinel) {
         const long long m_val = (long long)before + (u ? 1 : 0);
         if constexpr (kMode == kEmitAll) {
           for (long long v = s + 1; v <= n; v++) off[v] = m_val;
@@ -596,7 +558,7 @@ __global__ void __launch_bounds__(kCsrBlock, 5) csr_emit(const unsigned long lon
         }
       }
     }
-    running += tile_total;
+    t.step();
   }
 }
 
@@ -648,7 +610,8 @@ __global__ void csr_fill_starts(const long long* __restrict__ tail, long long n,
 // neighbour, and v's list opens with them.
 __global__ void csr_lower_emit(const unsigned long long* __restrict__ Bq, long long E, int B,
                                const long long* __restrict__ off, const unsigned long long* __restrict__ starts,
-                               int* __restrict__ adj) {
+                               int* __restrict__ adj, const long long* __restrict__ gv, long long G) {
+  GraphBase gb(gv, G);
   constexpr int kU = 4;  // keys per thread per step, all loaded first, then all their lookups
   const unsigned long long mask = (1ull << B) - 1;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -666,7 +629,11 @@ __global__ void csr_lower_emit(const unsigned long long* __restrict__ Bq, long l
     }
 #pragma unroll
     for (int u = 0; u < kU; u++)
-      if (x[u] != kSentinel) adj[at[u] + (unsigned long long)(i0 + u * stride)] = (int)(x[u] >> B);
+      if (x[u] != kSentinel) {
+        long long id = (long long)(x[u] >> B);
+        if (gv) id -= gb.of(id);
+        adj[at[u] + (unsigned long long)(i0 + u * stride)] = (int)id;
+      }
   }
 }
 
@@ -687,31 +654,45 @@ static int bits_for(long long n) {
   return B;
 }
 
-CsrLayout csr_layout(long long n, long long E, int sms, long long max_graph_n) {
+CsrLayout csr_layout(long long n, long long E, int sms, long long max_graph_n, bool allow_edges) {
   CsrLayout L{};
   long long N = 2 * E;
-  // five CTAs per SM, each sorting 2,048-key tiles with the next tile copied
-  // into shared memory while the current one is ranked (43 KB of shared
-  // memory, which admits five; registers held to five CTAs' worth by the
-  // kernels' launch bounds): resident warps and loads in flight count. Measured on R-MAT 24 (ms per build): 2 CTAs x
-  // 4,096-key tiles 56.8, 4 x 4,096 37.7, 6 x 2,048 35.6, 7 x 2,048 38.2,
-  // 8 x 1,536 37.3; with the asynchronous copy 5 x 2,048 31.0, 4 x 2,048 31.8
-  long long G = (long long)sms * 5;
-  long long tiles = (N + kTile - 1) / kTile;
-  if (tiles < G) G = tiles < 1 ? 1 : tiles;
-  L.grid = (int)G;
-  auto chunk_of = [&](long long keys) {
-    long long c = (keys + G - 1) / G;
-    c = (c + kTile - 1) / kTile * kTile;
-    return c < kTile ? (long long)kTile : c;
-  };
-  L.chunk = chunk_of(N);
-  L.chunk1 = chunk_of(E);
   L.N = N;
   L.Bs = bits_for(n);
   // batched: one spare code so that no valid (local) target has all bits set
   // and a valid key can never equal the sentinel in the sorted bits
   L.B = max_graph_n > 0 ? bits_for(max_graph_n + 1) : L.Bs;
+  // A single graph takes the edge route, a batch the route with fewer keys to
+  // move: 2B + B digit passes over E edge keys with global ids, or one sort of
+  // 2E arcs by (global source, local target). 256 graphs of 1k..200k vertices
+  // (139 M edges; 9 passes over E against 6 over 2E): 14.1 ms by arcs, 12.9 ms
+  // by edges.
+  const int edge_passes = (2 * L.Bs + 7) / 8 + (L.Bs + 7) / 8, arc_passes = (L.Bs + L.B + 7) / 8;
+  L.by_edges = max_graph_n <= 0 || (allow_edges && edge_passes < 2 * arc_passes);
+  if (L.by_edges) L.B = L.Bs;
+  // Three CTAs per SM (80 registers per thread), each sorting 4,096-key tiles:
+  // 16 keys per thread share a tile's barriers and its scan of the counters.
+  // Measured on 67 M random 44-bit keys (us per downsweep): 2,048-key tiles
+  // ranked by match.any, five CTAs 512; ranked through shared memory: 8 keys
+  // per thread, five CTAs 390, six 455 (spills); 12 keys, four CTAs 325; 14
+  // keys, four 335 (spills); 16 keys, three 305; ballots in place of the
+  // shared-memory masks 350.
+  // (1,024-key tiles for a list of less than one 4,096-key tile per CTA: 0.332
+  // against 0.318 ms for 1.0 M edges, not kept.)
+  const long long keys = L.by_edges ? E : N;
+  auto ctas_of = [&](long long k) {
+    return std::max<long long>(1, std::min<long long>((long long)sms * 3, (k + kSortTile - 1) / kSortTile));
+  };
+  const long long G = ctas_of(keys);
+  L.grid = (int)G;
+  L.chunk = std::max<long long>(1, (keys + G * kSortTile - 1) / (G * kSortTile)) * kSortTile;
+  // unique-key passes: a chunk of whole 256-key tiles per warp, eight CTAs per SM
+  auto warps_of = [&](long long k) {
+    return std::max<long long>(1, std::min<long long>((long long)sms * 64, (k + kUTile - 1) / kUTile));
+  };
+  const long long warps = warps_of(keys);
+  L.ugrid = (int)((warps + kCsrBlock / 32 - 1) / (kCsrBlock / 32));
+  L.uchunk = std::max<long long>(1, (keys + warps * kUTile - 1) / (warps * kUTile)) * kUTile;
   size_t off = 0;
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   L.status = off;
@@ -723,14 +704,16 @@ CsrLayout csr_layout(long long n, long long E, int sms, long long max_graph_n) {
   off = al(off + 8 * (size_t)(N + 2));
   L.keys1 = off;
   off = al(off + 8 * (size_t)(N + 2));
+  // sized for 2E keys on either route: a batch's workspace is at most a single graph's
+  const size_t counts = std::max<size_t>(256 * (size_t)ctas_of(N), (size_t)warps_of(N) + kCsrBlock / 32);
   L.hist = off;
-  off = al(off + 4 * 256 * (size_t)G);
+  off = al(off + 4 * counts);
   L.offs = off;
-  off = al(off + 8 * 256 * (size_t)G);
+  off = al(off + 8 * counts);
   L.rowtot = off;
   off = al(off + 8 * 256);
-  L.starts = off;  // a single graph's build: starts of the lower-neighbour lists
-  off = al(off + (max_graph_n > 0 ? 8 : 8 * (size_t)(n + 1)));
+  L.starts = off;  // the edge route: starts of the lower-neighbour lists
+  off = al(off + (L.by_edges ? 8 * (size_t)(n + 1) : 8));
   L.total = off;
   return L;
 }
@@ -751,8 +734,7 @@ cudaError_t csr_build_launch(const CsrLayout& L, char* ws, long long n, long lon
   if (E == 0) return cudaSuccess;
   const int G = L.grid;
   const EdgeList es{src, dst, n, L.B, gv, eoff, ngraphs, status};
-  // one radix pass: upsweep, row scans, downsweep (32-bit positions when the
-  // keys number at most 2^32)
+  // one radix pass: upsweep, row scans, downsweep
   auto pass = [&](int src_kind, const unsigned long long* in, unsigned long long* out, long long N, long long chunk,
                   int shift, int dmask) {
 #define KC_UP(S) rs_upsweep<S><<<G, kCsrBlock, 0, stream>>>(in, es, N, chunk, shift, dmask, hist)
@@ -760,22 +742,30 @@ cudaError_t csr_build_launch(const CsrLayout& L, char* ws, long long n, long lon
       case kKeys: KC_UP(kKeys); break;
       case kArcs: KC_UP(kArcs); break;
       case kCanon: KC_UP(kCanon); break;
+      case kCanonB: KC_UP(kCanonB); break;
       default: KC_UP(kKeysDrop); break;
     }
 #undef KC_UP
     scan_u32_to_u64<<<256, 1024, 0, stream>>>(hist, offs, G, rowtot);
+    // 32-bit positions when the keys number at most 2^32
     const bool narrow = N <= (1ll << 32);
-#define KC_DOWN(S, P) rs_downsweep<S, P><<<G, kCsrBlock, 0, stream>>>(in, es, out, N, chunk, shift, dmask, offs, rowtot)
+#define KC_RUN(S, P) rs_downsweep<S, P><<<G, kCsrBlock, 0, stream>>>(in, es, out, N, chunk, shift, dmask, offs, rowtot)
+#define KC_DOWN(S)                    \
+  if (narrow) KC_RUN(S, unsigned);    \
+  else KC_RUN(S, unsigned long long); \
+  break
     switch (src_kind) {
-      case kKeys: narrow ? KC_DOWN(kKeys, unsigned) : KC_DOWN(kKeys, unsigned long long); break;
-      case kArcs: narrow ? KC_DOWN(kArcs, unsigned) : KC_DOWN(kArcs, unsigned long long); break;
-      case kCanon: narrow ? KC_DOWN(kCanon, unsigned) : KC_DOWN(kCanon, unsigned long long); break;
-      default: narrow ? KC_DOWN(kKeysDrop, unsigned) : KC_DOWN(kKeysDrop, unsigned long long); break;
+      case kKeys: KC_DOWN(kKeys);
+      case kArcs: KC_DOWN(kArcs);
+      case kCanon: KC_DOWN(kCanon);
+      case kCanonB: KC_DOWN(kCanonB);
+      default: KC_DOWN(kKeysDrop);
     }
+#undef KC_RUN
 #undef KC_DOWN
   };
-  if (!gv) {
-    // a single graph: A = the E edge keys sorted by (min, max); B = A stably
+  if (L.by_edges) {
+    // the edge route: A = the E edge keys sorted by (min, max); B = A stably
     // sorted by max. A ping-pongs between the first halves of the two key
     // buffers, B between their second halves (from an even index: 16-byte
     // copies stay aligned)
@@ -783,7 +773,7 @@ cudaError_t csr_build_launch(const CsrLayout& L, char* ws, long long n, long lon
     unsigned long long *a0 = k0, *a1 = k1, *b0 = k0 + off2, *b1 = k1 + off2;
     const int passes_a = (2 * L.B + 7) / 8;
     for (int p = 0; p < passes_a; p++) {
-      pass(p == 0 ? kCanon : kKeys, a0, a1, E, L.chunk1, 8 * p, 0xff);
+      pass(p == 0 ? (gv ? kCanonB : kCanon) : kKeys, a0, a1, E, L.chunk, 8 * p, 0xff);
       std::swap(a0, a1);
     }
     const unsigned long long* A = a0;
@@ -793,7 +783,7 @@ cudaError_t csr_build_launch(const CsrLayout& L, char* ws, long long n, long lon
     const int passes_b = (L.B + 7) / 8;
     for (int p = 0; p < passes_b; p++) {
       const int bits = std::min(8, L.B - 8 * p);
-      pass(p == 0 ? kKeysDrop : kKeys, p == 0 ? A : b0, b1, E, L.chunk1, 8 * p, (1 << bits) - 1);
+      pass(p == 0 ? kKeysDrop : kKeys, p == 0 ? A : b0, b1, E, L.chunk, 8 * p, (1 << bits) - 1);
       std::swap(b0, b1);
     }
     const unsigned long long* Bq = b0;
@@ -806,25 +796,25 @@ cudaError_t csr_build_launch(const CsrLayout& L, char* ws, long long n, long lon
     if ((e = cudaMemsetAsync(starts, 0, 8 * (size_t)(n + 1), stream)) != cudaSuccess) return e;
     csr_lower_starts<<<key_grid, kCsrBlock, 0, stream>>>(Bq, E, L.B, n, starts, tail);
     csr_fill_starts<<<fill_grid, kCsrBlock, 0, stream>>>(tail, n, starts);
-    csr_count_unique<<<G, kCsrBlock, 0, stream>>>(A, E, L.chunk1, hist);
-    scan_u32_to_u64<<<1, 1024, 0, stream>>>(hist, offs, G, nullptr);
-    csr_emit<kEmitUpper><<<G, kCsrBlock, 0, stream>>>(A, E, L.chunk1, L.B, n, offs, adj_out, off_out, m_out,
-                                                     starts, tail);
+    csr_count_unique<<<L.ugrid, kCsrBlock, 0, stream>>>(A, E, L.uchunk, hist);
+    scan_u32_to_u64<<<1, 1024, 0, stream>>>(hist, offs, L.ugrid * (kCsrBlock / 32), nullptr);
+    csr_emit<kEmitUpper><<<L.ugrid, kCsrBlock, 0, stream>>>(A, E, L.uchunk, L.B, n, offs, adj_out, off_out, m_out,
+                                                     starts, tail, gv, ngraphs);
     csr_finish_offsets<<<fill_grid, kCsrBlock, 0, stream>>>(tail, n, off_out, starts);
-    csr_lower_emit<<<key_grid, kCsrBlock, 0, stream>>>(Bq, E, L.B, off_out, starts, adj_out);
+    csr_lower_emit<<<key_grid, kCsrBlock, 0, stream>>>(Bq, E, L.B, off_out, starts, adj_out, gv, ngraphs);
     return cudaGetLastError();
   }
-  // a batch: two arcs per edge, sorted by (global source, local target)
+  // the arc route: two arcs per edge, sorted by (global source, local target)
   const long long N = L.N;
   const int passes = (L.Bs + L.B + 7) / 8;
   for (int p = 0; p < passes; p++) {
     pass(p == 0 ? kArcs : kKeys, k0, k1, N, L.chunk, 8 * p, 0xff);
     std::swap(k0, k1);
   }
-  csr_count_unique<<<G, kCsrBlock, 0, stream>>>(k0, N, L.chunk, hist);
-  scan_u32_to_u64<<<1, 1024, 0, stream>>>(hist, offs, G, nullptr);
-  csr_emit<kEmitAll><<<G, kCsrBlock, 0, stream>>>(k0, N, L.chunk, L.B, n, offs, adj_out, off_out, m_out, nullptr,
-                                                  nullptr);
+  csr_count_unique<<<L.ugrid, kCsrBlock, 0, stream>>>(k0, N, L.uchunk, hist);
+  scan_u32_to_u64<<<1, 1024, 0, stream>>>(hist, offs, L.ugrid * (kCsrBlock / 32), nullptr);
+  csr_emit<kEmitAll><<<L.ugrid, kCsrBlock, 0, stream>>>(k0, N, L.uchunk, L.B, n, offs, adj_out, off_out, m_out, nullptr,
+                                                  nullptr, nullptr, 0);
   return cudaGetLastError();
 }
 
