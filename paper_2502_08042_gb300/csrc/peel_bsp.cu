@@ -58,6 +58,12 @@ constexpr int kHold = kWarp;
 constexpr int kStage = kWarp * kIlp + kHold;
 constexpr int kStageS = 128;
 constexpr int kPrefetchSlices = 256;  // appends of at most this many slices prefetch their arcs
+// Passes of at most this many items read the neighbours' offsets beside their
+// decrements (measured, R-MAT 20 / R-MAT 24 / ER-10k, ms: never 4.48 / 12.60 /
+// 0.149, 256 items 4.41 / 12.66 / 0.151, 1,024 4.31 / 12.59 / 0.138, 2,048 4.27
+// / 12.54 / 0.139, any pass 4.26 / 12.70 / 0.138: with more items the extra
+// reads miss L2).
+constexpr unsigned kEarlyItems = 2048;
 constexpr int kLenShift = 40;  // item = first arc | length << 40
 constexpr unsigned long long kArcMask = (1ull << kLenShift) - 1;
 // barrier word: arrivals in bits 0..30, the phase's queue appends in bits
@@ -81,8 +87,7 @@ struct Shared {
     int stage[kBlock * kTile];                      // scans (local queues are empty): frontier ids
   };
   int lqn[kWarps];
-  int part_i[kWarps];
-  int total_i;
+  int part_i[2][kWarps];
   unsigned long long base_a, base_q;
   int red_min[kWarps];
   int red_cnt[kWarps];
@@ -155,26 +160,36 @@ __device__ __forceinline__ unsigned long long make_item(long long a0, long long 
   return (unsigned long long)a0 | ((unsigned long long)len << kLenShift);
 }
 
-// Writes each lane's arc range [e0, e1), cut in `cnt` slices, to the queue
-// from slot p on. A lane with a few slices writes its own; the slices of a
-// long range (a hub) are written by the whole warp, so one lane never stores
-// thousands of items alone. Warp-collective.
+// Writes each lane's arc range [e0, e1), cut in `cnt` slices, to the queue:
+// the warp's tot slices go to p0 on, this lane's after excl of them. Lanes with
+// a slice or two each write their own; else the slices are spread over the
+// warp (a slice's lane by a search over the lanes' excl), so a hub's are not
+// stored by one lane and the stores are consecutive. Warp-collective.
 __device__ __forceinline__ void write_slices(const PeelArgs& a, long long e0, long long e1, int cnt,
-                                             unsigned long long p, int lane) {
-  constexpr int kOwn = 4;
-  if (cnt <= kOwn)
-    for (int i = 0; i < cnt; i++) {
-      const long long s0 = e0 + (long long)i * a.slice;
-      a.Q[p + i] = make_item(s0, min((long long)a.slice, e1 - s0));
+                                             unsigned long long p0, int excl, int tot, int lane) {
+  const bool pf = tot <= kPrefetchSlices;
+  if (!__any_sync(kFull, cnt > 2)) {
+    if (cnt > 0) {
+      a.Q[p0 + excl] = make_item(e0, min((long long)a.slice, e1 - e0));
+      if (pf) prefetch_arcs(a, e0);
     }
-  for (unsigned big = __ballot_sync(kFull, cnt > kOwn); big; big &= big - 1) {
-    const int L = __ffs(big) - 1;
+    if (cnt > 1) {
+      a.Q[p0 + excl + 1] = make_item(e0 + a.slice, e1 - e0 - a.slice);
+      if (pf) prefetch_arcs(a, e0 + a.slice);
+    }
+    return;
+  }
+  for (int j0 = 0; j0 < tot; j0 += kWarp) {
+    const int j = j0 + lane;
+    int L = 0;  // the last lane with excl <= j holds slice j
+#pragma unroll
+    for (int s = kWarp / 2; s > 0; s >>= 1)
+      if (__shfl_sync(kFull, excl, L + s) <= j) L += s;
     const long long b0 = __shfl_sync(kFull, e0, L), b1 = __shfl_sync(kFull, e1, L);
-    const unsigned long long bp = __shfl_sync(kFull, p, L);
-    const int bc = __shfl_sync(kFull, cnt, L);
-    for (int i = lane; i < bc; i += kWarp) {
-      const long long s0 = b0 + (long long)i * a.slice;
-      a.Q[bp + i] = make_item(s0, min((long long)a.slice, b1 - s0));
+    const long long s0 = b0 + (long long)(j - __shfl_sync(kFull, excl, L)) * a.slice;
+    if (j < tot) {
+      a.Q[p0 + j] = make_item(s0, min((long long)a.slice, b1 - s0));
+      if (pf) prefetch_arcs(a, s0);
     }
   }
 }
@@ -329,22 +344,20 @@ struct ScanOut {
   int dmin;
 };
 
-// Block-wide exclusive prefix sum of x; *total receives the block's sum.
-// Ends with every thread past the barrier that published the partial sums.
-__device__ __forceinline__ int block_excl_scan(Shared& sh, int x, int* total) {
+// Exclusive prefix sum over the CTA's warps of each warp's x; *total receives
+// the sum. One barrier: every warp scans the warps' sums itself, and the sums
+// alternate between two arrays (ph, toggled here), so the next call's stores
+// cannot meet this one's loads.
+__device__ __forceinline__ int block_excl_warps(Shared& sh, int& ph, int x, int* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int incl = warp_incl_scan(x, lane);
-  if (lane == 31) sh.part_i[warp] = incl;
+  int* part = sh.part_i[ph];
+  ph ^= 1;
+  if (lane == 0) part[warp] = x;
   __syncthreads();
-  if (warp == 0) {
-    const int y = lane < kWarps ? sh.part_i[lane] : 0;
-    const int yi = warp_incl_scan(y, lane);
-    if (lane < kWarps) sh.part_i[lane] = yi - y;
-    if (lane == kWarps - 1) sh.total_i = yi;
-  }
-  __syncthreads();
-  *total = sh.total_i;
-  return sh.part_i[warp] + incl - x;
+  const int y = lane < kWarps ? part[lane] : 0;
+  const int yi = warp_incl_scan(y, lane);
+  *total = __shfl_sync(kFull, yi, kWarps - 1);
+  return __shfl_sync(kFull, yi - y, warp);
 }
 
 // Scan of active-list entries [lo, hi) by one CTA: entries with d~ > keep_above
@@ -373,17 +386,25 @@ __device__ ScanOut scan_range(const PeelArgs& a, Shared& sh, RoundRec* R, unsign
   // level take_at for taken ones, nothing for kept ones)
   if (take_val < 0) take_val = take_at;
   const int tid = threadIdx.x;
+  const unsigned lt = lanemask_lt();
+  int ph = 0;                    // block_excl_warps' array in turn
   unsigned long long found = 0;  // staged frontier vertices (block-uniform)
   int direct = 0;                // frontier vertices without arcs (this thread)
   int nsampled = 0;              // first scan with sampling: vertices put in sample mode
   int dmin = INT_MAX;
   for (long long tile = lo; tile < hi; tile += (long long)kBlock * kTile) {
+    // a warp takes consecutive entries of the tile, 32 per slot (a short tile
+    // fills fewer slots, not fewer warps), so its loads and the stores of what
+    // it keeps are consecutive
+    const int rows = (int)min((long long)kTile, (hi - tile + kBlock - 1) / kBlock);
+    const int seg = (tid >> 5) * (kWarp * rows) + (tid & 31);
+    const long long end = min(hi, tile + (long long)kBlock * rows);
     int v[kTile];
     unsigned keep = 0, take = 0, over = 0, rec = 0;
 #pragma unroll
     for (int q = 0; q < kTile; q++) {
-      const long long i = tile + (long long)q * kBlock + tid;
-      v[q] = i < hi ? (Ain ? ld_once_s32(Ain + i, l2_evict_first_policy()) : (int)i) : -1;
+      const long long i = tile + seg + q * kWarp;
+      v[q] = q < rows && i < end ? (Ain ? ld_once_s32(Ain + i, l2_evict_first_policy()) : (int)i) : -1;
     }
     // the d~ of the tile's entries, every load issued before any is used (a
     // check that can branch between two loads makes each wait for the one
@@ -394,7 +415,7 @@ __device__ ScanOut scan_range(const PeelArgs& a, Shared& sh, RoundRec* R, unsign
 #pragma unroll
       for (int q = 0; q < kTile; q++) {
         const bool in = (unsigned)v[q] < (unsigned)a.n;
-        bad |= !in && tile + (long long)q * kBlock + tid < hi;
+        bad |= !in && q < rows && tile + seg + q * kWarp < end;
         if (!in) v[q] = -1;
         d[q] = in ? __ldcg(a.deg + v[q]) : 0;
       }
@@ -471,35 +492,45 @@ __device__ ScanOut scan_range(const PeelArgs& a, Shared& sh, RoundRec* R, unsign
       }
     }
     // block-wide offsets of (kept, taken): kept entries go to Aout after one
-    // atomic per tile, taken ones to the shared-memory stage
+    // atomic per tile, taken ones to the shared-memory stage while it returns
     int tot;
-    const int ex = block_excl_scan(sh, (__popc(take) << 16) | __popc(keep), &tot);
+    const int at = block_excl_warps(
+        sh, ph, (int)__reduce_add_sync(kFull, (unsigned)((__popc(take) << 16) | __popc(keep))), &tot);
     if (tid == 0) sh.base_a = (tot & 0xffff) ? atomicAdd(&R->alen, (unsigned long long)(tot & 0xffff)) : 0;
-    __syncthreads();
-    unsigned long long pa = sh.base_a + (ex & 0xffff);
-    int ps = ex >> 16;
+    int ps = at >> 16;
 #pragma unroll
     for (int q = 0; q < kTile; q++) {
-      if ((keep >> q) & 1u) st_once_s32(Aout + pa++, v[q], l2_evict_first_policy());
-      if ((take >> q) & 1u) sh.stage[ps++] = v[q];
+      const unsigned m = __ballot_sync(kFull, (take >> q) & 1u);
+      if ((take >> q) & 1u) sh.stage[ps + __popc(m & lt)] = v[q];
+      ps += __popc(m);
+    }
+    __syncthreads();
+    int* kept = Aout + (Aout ? sh.base_a + (at & 0xffff) : 0);
+#pragma unroll
+    for (int q = 0; q < kTile; q++) {
+      const unsigned m = __ballot_sync(kFull, (keep >> q) & 1u);
+      if ((keep >> q) & 1u) st_once_s32(kept + __popc(m & lt), v[q], l2_evict_first_policy());
+      kept += __popc(m);
     }
     if (Aover) {
+      const int c = __popc(over), incl = warp_incl_scan(c, tid & 31);
       int otot;
-      const int oex = block_excl_scan(sh, __popc(over), &otot);
+      const int oat = block_excl_warps(sh, ph, __shfl_sync(kFull, incl, 31), &otot);
       if (tid == 0) sh.base_q = otot ? atomicAdd(&R->head, (unsigned long long)otot) : 0;
       __syncthreads();
-      unsigned long long po = sh.base_q + oex;
+      unsigned long long po = sh.base_q + oat + incl - c;
 #pragma unroll
       for (int q = 0; q < kTile; q++)
         if ((over >> q) & 1u) Aover[po++] = v[q];
+      __syncthreads();
     }
-    __syncthreads();
     const int ntaken = tot >> 16;
     found += ntaken;
     // expand the staged frontier vertices into slices, kExpand per thread per round
     for (int base = 0; base < ntaken; base += kBlock * kExpand) {
+      // (a warp's slots go to the queue one after another)
       long long e0[kExpand], e1[kExpand];
-      int nsl = 0;
+      int excl[kExpand], wtot[kExpand + 1];
 #pragma unroll
       for (int k = 0; k < kExpand; k++) {
         const int i = base + k * kBlock + tid;
@@ -512,10 +543,16 @@ __device__ ScanOut scan_range(const PeelArgs& a, Shared& sh, RoundRec* R, unsign
           if constexpr (kSample) a.stamp[x] = stamp_val;
         }
       }
+      wtot[0] = 0;
 #pragma unroll
-      for (int k = 0; k < kExpand; k++) nsl += slices_of(a, e0[k], e1[k]);
+      for (int k = 0; k < kExpand; k++) {
+        const int c = slices_of(a, e0[k], e1[k]);
+        const int incl = warp_incl_scan(c, tid & 31);
+        excl[k] = incl - c;
+        wtot[k + 1] = wtot[k] + __shfl_sync(kFull, incl, 31);
+      }
       int ntot;
-      const int exs = block_excl_scan(sh, nsl, &ntot);
+      const int wbase = block_excl_warps(sh, ph, wtot[kExpand], &ntot);
       if (tid == 0) {
         unsigned long long bq = qbase + (ntot ? atomicAdd(&R->tail, (unsigned long long)ntot) : 0);
         s_app += (unsigned long long)ntot;
@@ -527,13 +564,13 @@ __device__ ScanOut scan_range(const PeelArgs& a, Shared& sh, RoundRec* R, unsign
       }
       __syncthreads();
       if (sh.base_q != ~0ull) {
-        unsigned long long pq = sh.base_q + exs;
 #pragma unroll
-        for (int k = 0; k < kExpand; k++)
-          for (long long s0 = e0[k]; s0 < e1[k]; s0 += a.slice) {
-            a.Q[pq++] = make_item(s0, min((long long)a.slice, e1[k] - s0));
-            if (ntot <= kPrefetchSlices) prefetch_arcs(a, s0);
-          }
+        for (int k = 0; k < kExpand; k++) {
+          const int tot = wtot[k + 1] - wtot[k];
+          if (tot)
+            write_slices(a, e0[k], e1[k], slices_of(a, e0[k], e1[k]), sh.base_q + wbase + wtot[k], excl[k], tot,
+                         tid & 31);
+        }
       }
       __syncthreads();
     }
@@ -576,11 +613,11 @@ struct PassCtx {
   int* near;                // the active list, appended from near_base on (count in R->found)
   unsigned long long near_base;
   int pass;                 // sampling: index of the running pass (stamps)
+  bool early;               // short pass: read offsets beside decrements (see process_items)
 };
 
 // Appends `cnt` items per lane (lane-owned arc ranges [e0, e1) cut in
 // slices) to the queue.
-template <bool kCoop = false>
 __device__ __forceinline__ void append_ranges(const PeelArgs& a, const PassCtx& pc, int cnt, long long e0,
                                               long long e1, int lane) {
   const int incl = warp_incl_scan(cnt, lane);
@@ -596,32 +633,19 @@ __device__ __forceinline__ void append_ranges(const PeelArgs& a, const PassCtx& 
     if (lane == 0) raise_status(a, ST_CAPACITY);
     return;
   }
-  unsigned long long p = base + (unsigned long long)(incl - cnt);
-  if constexpr (kCoop) {
-    write_slices(a, e0, e1, cnt, p, lane);
-  } else {
-    for (long long s0 = e0; s0 < e1 && cnt > 0; s0 += a.slice) {
-      a.Q[p++] = make_item(s0, min((long long)a.slice, e1 - s0));
-      if (tot <= kPrefetchSlices) prefetch_arcs(a, s0);
-    }
-  }
+  write_slices(a, e0, e1, cnt, base, incl - cnt, tot, lane);
 }
 
 // The vertices u of the lanes with `flag` crossed to the current level (their
-// coreness is set): one-slice lists go to the warp's local queue while it has
-// room, the rest go to the queue as slices for the next pass.
+// coreness is set) and own the arcs [e0, e1): one-slice lists go to the warp's
+// local queue while it has room, the rest go to the queue as slices for the
+// next pass.
 template <bool kSample = false>
-__device__ __forceinline__ void push_crossed(const PeelArgs& a, ShT<kSample>& sh, const PassCtx& pc, bool flag,
-                                             int u, int warp, int lane) {
-  long long e0 = 0, e1 = 0;
-  int nsl = 0;
-  if (flag) {
-    e0 = __ldcs(a.off + u);
-    e1 = __ldcs(a.off + u + 1);
-    nsl = slices_of(a, e0, e1);
-    // its first adjacency line is read next, here or by another warp
-    if (e1 > e0) prefetch_arcs(a, e0);
-  }
+__device__ __forceinline__ void push_ranges(const PeelArgs& a, ShT<kSample>& sh, const PassCtx& pc, bool flag, int u,
+                                            long long e0, long long e1, int warp, int lane) {
+  const int nsl = flag ? slices_of(a, e0, e1) : 0;
+  // its first adjacency line is read next, here or by another warp
+  if (nsl) prefetch_arcs(a, e0);
   const bool one = flag && nsl == 1;
   const unsigned om = __ballot_sync(kFull, one);
   const int lqn = sh.lqn[warp];
@@ -638,6 +662,17 @@ __device__ __forceinline__ void push_crossed(const PeelArgs& a, ShT<kSample>& sh
   if (lane == 0) sh.lqn[warp] = lqn + min(__popc(om), room);
   __syncwarp();
   append_ranges(a, pc, (flag && !local) ? nsl : 0, e0, e1, lane);
+}
+
+template <bool kSample = false>
+__device__ __forceinline__ void push_crossed(const PeelArgs& a, ShT<kSample>& sh, const PassCtx& pc, bool flag,
+                                             int u, int warp, int lane) {
+  long long e0 = 0, e1 = 0;
+  if (flag) {
+    e0 = __ldcs(a.off + u);
+    e1 = __ldcs(a.off + u + 1);
+  }
+  push_ranges<kSample>(a, sh, pc, flag, u, e0, e1, warp, lane);
 }
 
 // Pushes the nx vertices staged in sh.xs[warp], 32 at a time. Warp-collective.
@@ -722,6 +757,39 @@ __device__ void process_items(const PeelArgs& a, ShT<kSample>& sh, const PassCtx
   const int t = pc.t;
   const ArcMap mp = map_items(a, sh, item, c, warp, lane);
   const int total = mp.total;
+  if constexpr (!kWin && !kSample && !kCombine) {
+    // A batch of one window in a short pass, the common one of a long peel: its
+    // neighbours' offsets are read beside their decrements, not after them,
+    // so a crossing saves one round trip of the phase's chain.
+    if (total <= kWarp && pc.early) {
+      int u = -1, old = INT_MIN, none = 0;
+      const long long arc = mp.arc(0, lane, none);
+      if (lane < total) u = ld_stream_s32(a.adj + arc);
+      const bool in = (unsigned)u < (unsigned)a.n;
+      long long e0 = 0, e1 = 0;
+      if (in) {
+        old = atomicSub(a.deg + u, 1);
+        e0 = __ldcs(a.off + u);
+        e1 = __ldcs(a.off + u + 1);
+      }
+      if (lane < total && !in) raise_status(a, ST_NOT_SIMPLE);
+      const bool cross = old == t + 1;
+      const unsigned cm = __ballot_sync(kFull, cross);
+      if (cm) {
+        if (cross) a.core[u] = pc.val;
+        push_ranges(a, sh, pc, cross, u, e0, e1, warp, lane);
+      }
+      if (lane == 0) {
+        if (a.threshold) sh.ncross[warp] += __popc(cm);
+        if (a.trace) {
+          sh.tr_arcs[warp] += total;
+          sh.tr_decs[warp] += total;
+        }
+      }
+      __syncwarp();
+      return;
+    }
+  }
   int ndec = 0;
   unsigned nheads = 0;
   int nx = 0;             // crossing vertices staged (warp-uniform)
@@ -1050,7 +1118,7 @@ __device__ void run_apply(const PeelArgs& a, const PassCtx& pc, const int* list,
         raise_status(a, ST_CAPACITY);
       }
     }
-    append_ranges<true>(a, pc, cross ? nsl : 0, e0, e1, lane);
+    append_ranges(a, pc, cross ? nsl : 0, e0, e1, lane);
   }
 }
 
@@ -1147,7 +1215,7 @@ __device__ void run_recount_apply(const PeelArgs& a, const PassCtx& pc, unsigned
     const unsigned jm = __ballot_sync(kFull, join);
     if (jm && lane == 0) atomicAdd(&pc.R->found, (unsigned long long)__popc(jm));
     const int nsl = join ? slices_of(a, e0, e1) : 0;
-    append_ranges<true>(a, pc, nsl, e0, e1, lane);
+    append_ranges(a, pc, nsl, e0, e1, lane);
   }
   kmin = warp_min(kmin);
   if (lane == 0 && kmin != INT_MAX) atomicMax(&pc.R->minkey, INT_MAX - kmin);
@@ -1574,7 +1642,7 @@ __global__ void __launch_bounds__(kBlock, 2) peel_bsp(PeelArgs a) {
       // warp; R-MAT passes a few)
       const bool pre = (qend - qb) >= (unsigned long long)a.precheck_items * nctas * kWarps;
       const PassCtx pc{P, qend, t, a.threshold ? 0 : t, pre, W ? hi_w : -1, const_cast<int*>(Acur),
-                       (unsigned long long)(la + near_extra)};
+                       (unsigned long long)(la + near_extra), 0, qend - qb <= kEarlyItems};
       run_pass<kWindow, false, kCombine>(a, sh, pc, qb, qend, solo ? 0 : (int)blockIdx.x, nctas);
       if (a.threshold && lane == 0 && sh.ncross[warp]) {
         atomicAdd(&a.ctl->crossed, (unsigned long long)sh.ncross[warp]);
