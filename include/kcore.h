@@ -253,7 +253,7 @@ kcore_status kcore_decompose_host(kcore_handle h, int64_t n, int64_t m, const in
  *   6  symmetry: u in list(v) implies v in list(u) (binary search in list(u))
  *   n, m         vertices and arcs (0 <= n <= 2^31 - 2; m = 0 when n = 0)
  *   offsets, adj device int64[n+1], int32[m], borrowed, read only
- * Asynchronous: two kernels on `stream`, O(m log d_max) work. kcore_sync_status
+ * Asynchronous: three kernels on `stream`, O(m log d_max) work. kcore_sync_status
  * returns KCORE_OK for a simple CSR, else KCORE_ERR_NOT_SIMPLE with the first
  * failure recorded (which one, when several threads fail at once, is
  * unspecified) in kcore_stats.invalid_check / invalid_vertex / invalid_arc and

@@ -212,7 +212,7 @@ cudaError_t bsp_barrier_probe(const PeelArgs& args, int grid, int iters, unsigne
 cudaError_t sample_check_launch(long long n, long long m, const long long* off, const int* adj, const int* core,
                                 int* acc, PeelCtl* ctl, int sms, cudaStream_t stream);
 
-// Simple-CSR check (validate.cu). st: device int[8] (code, pad, vertex, arc as
+// Simple-CSR check (validate.cu). st: device int[16] (code, pad, vertex, arc as
 // int64); zeroed by the launch, code 0 when the CSR is simple.
 cudaError_t validate_launch(long long n, long long m, const long long* off, const int* adj, int* st, int sms,
                             cudaStream_t stream);
