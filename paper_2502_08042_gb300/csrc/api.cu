@@ -403,10 +403,15 @@ kcore_status peel_call(kcore_ctx* h, int64_t n, int64_t m, const int64_t* offset
   const int mode = threshold ? 2 : effective_mode(h);
   const int slice =
       h->opt[KCORE_OPT_SLICE_ARCS] > 0 ? (int)h->opt[KCORE_OPT_SLICE_ARCS] : (mode == 1 ? 512 : kc::kSliceDefault);
-  const bool hybrid = mode == 2 && !threshold && h->opt[KCORE_OPT_BATCH_UPDATE] != 0 &&
-                      h->opt[KCORE_OPT_LEVEL_WINDOW] == 0;
+  bool hybrid = mode == 2 && h->opt[KCORE_OPT_BATCH_UPDATE] != 0 &&
+                (threshold || h->opt[KCORE_OPT_LEVEL_WINDOW] == 0);
   const bool sample = sampling_on(h, threshold);
   PeelLayout L = peel_layout(n, m, slice, mode == 3 || hybrid, sample);
+  if (threshold && h->ws_external && h->ws_bytes < L.total) {
+    // a caller's workspace without room for the counts: the query needs none
+    hybrid = false;
+    L = peel_layout(n, m, slice, false, sample);
+  }
   kcore_status st = ensure_ws(h, L.total);
   if (st != KCORE_OK) return st;
   char* ws = (char*)h->ws;
@@ -439,7 +444,7 @@ kcore_status peel_call(kcore_ctx* h, int64_t n, int64_t m, const int64_t* offset
   a.local_batches = h->opt[KCORE_OPT_LOCAL_BATCHES] > 0 ? (int)h->opt[KCORE_OPT_LOCAL_BATCHES] : INT32_MAX;
   a.threshold = threshold ? 1 : 0;
   a.offline = mode == 3 ? 1 : 0;
-  a.window = mode == 2 ? (int)h->opt[KCORE_OPT_LEVEL_WINDOW] : 0;
+  a.window = mode == 2 && !threshold ? (int)h->opt[KCORE_OPT_LEVEL_WINDOW] : 0;
   a.hybrid = hybrid ? 1 : 0;
   a.A2 = (int*)(ws + L.a2);
   a.hcnt = (int*)(ws + L.hcnt);
