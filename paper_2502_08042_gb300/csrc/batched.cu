@@ -760,186 +760,177 @@ struct ClusterPeel {
   }
 };
 
-// graph g of a batch: vertices [v0, v0 + n)
-__device__ __forceinline__ GraphDesc batch_desc(const BatchArgs& a, long long g, long long v0, long long n) {
-  return GraphDesc{a.off + v0, a.adj,     a.core + v0, a.kmax + g, a.deg + v0, a.A0 + v0,
-                   a.A1 + v0,  a.F0 + v0, a.F1 + v0,   n,          a.m};
-}
+// Where a kernel's graphs come from: a batch's segmented CSR, or descriptors in
+// a device table (graphs in separate allocations, as the server holds them;
+// the launch lists the table slots to process). find() looks up the graph at
+// position gi of the processing order, desc() describes it.
+struct Found {
+  long long g, v0, n, arcs;  // graph (or slot), first vertex, vertices, arcs
+};
+struct BatchSource {
+  const BatchArgs& a;
+  __device__ __forceinline__ long long count() const { return a.G; }
+  __device__ __forceinline__ int* next() const { return a.next_graph; }
+  __device__ __forceinline__ int* status() const { return a.status; }
+  __device__ __forceinline__ int smem() const { return a.smem_deg_max; }
+  __device__ __forceinline__ long long team_arcs() const { return a.team_arcs; }
+  // false: a failed check, recorded by the thread that reports it
+  __device__ __forceinline__ bool find(long long gi, bool report, int* bad, Found* f) const {
+    f->g = a.order ? a.order[gi] : gi;
+    if (f->g < 0 || f->g >= a.G) {  // the order is a permutation of [0, G); checked anyway
+      if (report) flag_bad(a.status, 8, f->g, bad);
+      return false;
+    }
+    f->v0 = a.gv[f->g];
+    f->n = a.gv[f->g + 1] - f->v0;
+    if (f->v0 < 0 || f->n < 0 || f->v0 + f->n > a.N) {  // graph outside the vertex range
+      if (report) {
+        flag_bad(a.status, 9, f->g, bad);
+        a.kmax[f->g] = -1;
+      }
+      return false;
+    }
+    f->arcs = a.off[f->v0 + f->n] - a.off[f->v0];
+    return true;
+  }
+  __device__ __forceinline__ GraphDesc desc(const Found& f) const {
+    return GraphDesc{a.off + f.v0, a.adj,       a.core + f.v0, a.kmax + f.g, a.deg + f.v0, a.A0 + f.v0,
+                     a.A1 + f.v0,  a.F0 + f.v0, a.F1 + f.v0,   f.n,          a.m};
+  }
+};
+struct ListSource {
+  const GraphDesc* table;
+  const SlotList& list;
+  int* next_;
+  int* status_;
+  int smem_deg_max;
+  long long team_arcs_;
+  __device__ __forceinline__ long long count() const { return list.count; }
+  __device__ __forceinline__ int* next() const { return next_; }
+  __device__ __forceinline__ int* status() const { return status_; }
+  __device__ __forceinline__ int smem() const { return smem_deg_max; }
+  __device__ __forceinline__ long long team_arcs() const { return team_arcs_; }
+  __device__ __forceinline__ bool find(long long gi, bool, int*, Found* f) const {
+    f->g = list.slot[gi];
+    const GraphDesc& d = table[f->g];
+    f->v0 = 0;
+    f->n = d.n;
+    f->arcs = d.n > 0 ? d.off[d.n] - d.off[0] : 0;
+    return true;
+  }
+  __device__ __forceinline__ GraphDesc desc(const Found& f) const { return table[f.g]; }
+};
 
 // Draws graph after graph for the team and peels them. first >= 0: a graph the
-// CTA drew already. With a.team_arcs > 0, returns the first graph below that
-// many arcs unpeeled (its position), else -1 once the batch is exhausted.
-template <int BLOCK>
-__device__ long long peel_drawn(const BatchArgs& a, int smem_deg_max, int* sdeg, BatchShared<BLOCK>& sh, long long first,
+// CTA drew already. With stop_below > 0, returns the position of the first
+// graph of fewer arcs, unpeeled; -1 once the graphs are exhausted.
+template <int BLOCK, typename Source>
+__device__ long long peel_drawn(const Source& src, int smem_deg_max, int* sdeg, BatchShared<BLOCK>& sh, long long first,
                                 long long stop_below) {
   const int tid = team_tid<BLOCK>();
   for (;;) {
-    if (tid == 0) sh.g = first >= 0 ? (int)first : atomicAdd(a.next_graph, 1);
+    if (tid == 0) sh.g = first >= 0 ? (int)first : atomicAdd(src.next(), 1);
     first = -1;
     team_sync<BLOCK>();
     const long long gi = sh.g;
     team_sync<BLOCK>();
-    if (gi >= a.G) return -1;
-    const long long g = a.order ? a.order[gi] : gi;
-    if (g < 0 || g >= a.G) {  // the order is a permutation of [0, G); checked anyway
-      if (tid == 0) flag_bad(a.status, 8, g, &sh.bad);
-      continue;
-    }
-    const long long v0 = a.gv[g], n = a.gv[g + 1] - v0;
-    if (v0 < 0 || n < 0 || v0 + n > a.N) {  // graph outside the vertex range
-      if (tid == 0) {
-        flag_bad(a.status, 9, g, &sh.bad);
-        a.kmax[g] = -1;
-      }
-      continue;
-    }
-    if (stop_below > 0 && a.off[v0 + n] - a.off[v0] < stop_below) return gi;
-    if (tid == 0) sh.gd = batch_desc(a, g, v0, n);
+    if (gi >= src.count()) return -1;
+    Found f;
+    if (!src.find(gi, tid == 0, &sh.bad, &f)) continue;
+    if (f.arcs < stop_below) return gi;
+    if (tid == 0) sh.gd = src.desc(f);
     team_sync<BLOCK>();
-    peel_one_graph<BLOCK>(smem_deg_max, a.status, sdeg, sh);
+    peel_one_graph<BLOCK>(smem_deg_max, src.status(), sdeg, sh);
   }
 }
 
-// A 1,024-thread CTA peels whole graphs while they are large (a.team_arcs arcs
+// A 1,024-thread CTA peels whole graphs while they are large (team_arcs arcs
 // or more; the order is by arcs) and from the first smaller one on splits into
 // teams of kTeam threads, each drawing graphs of its own with its share of the
 // shared memory: a small graph's phases are short dependent chains that leave
 // most of an SM idle.
 constexpr int kTeam = 512;
+template <int BLOCK>
+constexpr int kTeams = BLOCK >= 1024 ? BLOCK / kTeam : 1;
+template <int BLOCK>
+union CtaShared {
+  BatchShared<BLOCK> whole;
+  BatchShared<BLOCK / kTeams<BLOCK>> team[kTeams<BLOCK>];
+};
+template <int BLOCK, typename Source>
+__device__ void peel_cta(const Source& src, int* sdeg, CtaShared<BLOCK>& sh, long long first) {
+  constexpr int T = kTeams<BLOCK>;
+  const long long gi = peel_drawn<BLOCK>(src, src.smem(), sdeg, sh.whole, first, T > 1 ? src.team_arcs() : 0);
+  if constexpr (T > 1) {
+    if (gi < 0) return;
+    __syncthreads();
+    const int t = threadIdx.x / kTeam, share = src.smem() / T;
+    peel_drawn<kTeam>(src, share, sdeg + t * share, sh.team[t], t == 0 ? gi : -1, 0);
+  }
+}
+
+// The clustered form: clusters of C CTAs for the graphs of at least big_arcs
+// arcs (see the file comment). A cluster draws graphs together while they are
+// big; from the first graph below the threshold on, its CTAs draw their own
+// (the first CTA starts with that graph).
+template <int BLOCK, int C, typename Source>
+__device__ void peel_cluster(const Source& src, int* sdeg, CtaShared<BLOCK>& sh, ClusterCtl& ctl, long long big_arcs) {
+  cg::cluster_group cl = cg::this_cluster();
+  ClusterCtl* lc = cl.map_shared_rank(&ctl, 0);
+  const bool lead = cl.block_rank() == 0;
+  for (;;) {
+    if (lead && threadIdx.x == 0) ctl.g = atomicAdd(src.next(), 1);
+    cl.sync();
+    const long long gi = lc->g;
+    cl.sync();  // every CTA has read the draw before the next one
+    if (gi >= src.count()) return;
+    Found f;
+    if (!src.find(gi, lead && threadIdx.x == 0, &sh.whole.bad, &f)) continue;
+    if (!(f.n > 0 && f.n < INT_MAX && f.arcs >= big_arcs)) {
+      peel_cta<BLOCK>(src, sdeg, sh, lead ? gi : -1);
+      return;
+    }
+    if (threadIdx.x == 0) sh.whole.gd = src.desc(f);
+    __syncthreads();
+    ClusterPeel<BLOCK, C> cp(lc, sh.whole, src.status());
+    cp.peel(sh.whole.gd);
+  }
+}
 
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 2048 / BLOCK * 3 / 4)) batch_peel(BatchArgs a) {
   extern __shared__ int sdeg[];
-  constexpr int kTeams = BLOCK >= 1024 ? BLOCK / kTeam : 1;
-  __shared__ union {
-    BatchShared<BLOCK> whole;
-    BatchShared<BLOCK / kTeams> team[kTeams];
-  } sh;
-  long long gi = peel_drawn<BLOCK>(a, a.smem_deg_max, sdeg, sh.whole, -1, kTeams > 1 ? a.team_arcs : 0);
-  if constexpr (kTeams > 1) {
-    if (gi < 0) return;
-    __syncthreads();
-    const int t = threadIdx.x / kTeam, share = a.smem_deg_max / kTeams;
-    peel_drawn<kTeam>(a, share, sdeg + t * share, sh.team[t], t == 0 ? gi : -1, 0);
-  }
+  __shared__ CtaShared<BLOCK> sh;
+  peel_cta<BLOCK>(BatchSource{a}, sdeg, sh, -1);
 }
 
-// The batched peel with clusters of C CTAs for the graphs of at least big_arcs
-// arcs (see the file comment). A cluster draws graphs together while they are
-// big; from the first graph below the threshold on, its CTAs draw one each.
 template <int BLOCK, int C>
 __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 2048 / BLOCK / 2))
     batch_peel_cl(BatchArgs a, long long big_arcs) {
   extern __shared__ int sdeg[];
-  __shared__ BatchShared<BLOCK> sh;
+  __shared__ CtaShared<BLOCK> sh;
   __shared__ ClusterCtl ctl;
-  cg::cluster_group cl = cg::this_cluster();
-  ClusterCtl* lc = cl.map_shared_rank(&ctl, 0);
-  const bool lead = cl.block_rank() == 0;
-  bool together = true;
-  for (;;) {
-    long long gi;
-    if (together) {
-      if (lead && threadIdx.x == 0) ctl.g = atomicAdd(a.next_graph, 1);
-      cl.sync();
-      gi = lc->g;
-      cl.sync();  // every CTA has read the draw before the next one
-    } else {
-      if (threadIdx.x == 0) sh.g = atomicAdd(a.next_graph, 1);
-      __syncthreads();
-      gi = sh.g;
-      __syncthreads();
-    }
-    if (gi >= a.G) break;
-    const long long g = a.order ? a.order[gi] : gi;
-    if (g < 0 || g >= a.G) {
-      if (threadIdx.x == 0) flag_bad(a.status, 8, g, &sh.bad);
-      continue;
-    }
-    const long long v0 = a.gv[g], n = a.gv[g + 1] - v0;
-    if (v0 < 0 || n < 0 || v0 + n > a.N) {
-      if (threadIdx.x == 0 && (!together || lead)) {
-        flag_bad(a.status, 9, g, &sh.bad);
-        a.kmax[g] = -1;
-      }
-      continue;
-    }
-    if (threadIdx.x == 0) sh.gd = batch_desc(a, g, v0, n);
-    __syncthreads();
-    if (together && n > 0 && n < INT_MAX && a.off[v0 + n] - a.off[v0] >= big_arcs) {
-      ClusterPeel<BLOCK, C> cp(lc, sh, a.status);
-      cp.peel(sh.gd);
-      continue;
-    }
-    if (together) {
-      together = false;  // the first CTA peels this graph, the others draw their own
-      if (!lead) continue;
-    }
-    peel_one_graph<BLOCK>(a.smem_deg_max, a.status, sdeg, sh);
-  }
+  peel_cluster<BLOCK, C>(BatchSource{a}, sdeg, sh, ctl, big_arcs);
 }
 
-// The same peel over graph descriptors held in a device table (graphs in
-// separate allocations, as the server holds them). The launch lists the
-// table slots to process; CTAs take them from a counter.
+// (the launch lists the slots largest first)
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 2048 / BLOCK / 2))
-    desc_peel(const GraphDesc* table, SlotList list, int* next, int smem_deg_max, int* status) {
+    desc_peel(const GraphDesc* table, const __grid_constant__ SlotList list, int* next, int smem_deg_max, int* status,
+              long long team_arcs) {
   extern __shared__ int sdeg[];
-  __shared__ BatchShared<BLOCK> sh;
-  for (;;) {
-    if (threadIdx.x == 0) sh.g = atomicAdd(next, 1);
-    __syncthreads();
-    int gi = sh.g;
-    __syncthreads();
-    if (gi >= list.count) break;
-    if (threadIdx.x == 0) sh.gd = table[list.slot[gi]];
-    __syncthreads();
-    peel_one_graph<BLOCK>(smem_deg_max, status, sdeg, sh);
-  }
+  __shared__ CtaShared<BLOCK> sh;
+  peel_cta<BLOCK>(ListSource{table, list, next, status, smem_deg_max, team_arcs}, sdeg, sh, -1);
 }
 
-// The descriptor-driven peel with clusters of C CTAs for the graphs of at
-// least big_arcs arcs (the launch lists the slots largest first).
 template <int BLOCK, int C>
 __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 2048 / BLOCK / 2))
-    desc_peel_cl(const GraphDesc* table, SlotList list, int* next, int smem_deg_max, int* status,
-                 long long big_arcs) {
+    desc_peel_cl(const GraphDesc* table, const __grid_constant__ SlotList list, int* next, int smem_deg_max, int* status,
+                 long long team_arcs, long long big_arcs) {
   extern __shared__ int sdeg[];
-  __shared__ BatchShared<BLOCK> sh;
+  __shared__ CtaShared<BLOCK> sh;
   __shared__ ClusterCtl ctl;
-  cg::cluster_group cl = cg::this_cluster();
-  ClusterCtl* lc = cl.map_shared_rank(&ctl, 0);
-  const bool lead = cl.block_rank() == 0;
-  bool together = true;
-  for (;;) {
-    int gi;
-    if (together) {
-      if (lead && threadIdx.x == 0) ctl.g = atomicAdd(next, 1);
-      cl.sync();
-      gi = lc->g;
-      cl.sync();  // every CTA has read the draw before the next one
-    } else {
-      if (threadIdx.x == 0) sh.g = atomicAdd(next, 1);
-      __syncthreads();
-      gi = sh.g;
-      __syncthreads();
-    }
-    if (gi >= list.count) break;
-    if (threadIdx.x == 0) sh.gd = table[list.slot[gi]];
-    __syncthreads();
-    const GraphDesc& gd = sh.gd;
-    if (together && gd.n > 0 && gd.n < INT_MAX && gd.off[gd.n] - gd.off[0] >= big_arcs) {
-      ClusterPeel<BLOCK, C> cp(lc, sh, status);
-      cp.peel(gd);
-      continue;
-    }
-    if (together) {
-      together = false;  // the first CTA peels this graph, the others draw their own
-      if (!lead) continue;
-    }
-    peel_one_graph<BLOCK>(smem_deg_max, status, sdeg, sh);
-  }
+  peel_cluster<BLOCK, C>(ListSource{table, list, next, status, smem_deg_max, team_arcs}, sdeg, sh, ctl, big_arcs);
 }
 
 // Order of graphs: descending number of arcs (ties by index). One CTA sorts
@@ -1014,31 +1005,32 @@ int occupancy_block(size_t smem) {
 namespace {
 template <int C>
 cudaError_t desc_launch_cl(const GraphDesc* table, const SlotList& list, int* next, int smem_deg_max, int* status,
-                           int grid, size_t smem, long long big_arcs, cudaStream_t stream) {
+                           int grid, size_t smem, long long team_arcs, long long big_arcs, cudaStream_t stream) {
   cudaError_t e = cudaFuncSetAttribute(desc_peel_cl<1024, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
   grid = std::max(C, grid / C * C);
-  desc_peel_cl<1024, C><<<grid, 1024, smem, stream>>>(table, list, next, smem_deg_max, status, big_arcs);
+  desc_peel_cl<1024, C><<<grid, 1024, smem, stream>>>(table, list, next, smem_deg_max, status, team_arcs, big_arcs);
   return cudaGetLastError();
 }
 }  // namespace
 
 cudaError_t desc_launch(const GraphDesc* table, const SlotList& list, int* next, int smem_deg_max,
-                        int* status, int grid, size_t smem, cudaStream_t stream, int cluster, long long big_arcs) {
+                        int* status, int grid, size_t smem, cudaStream_t stream, long long team_arcs, int cluster,
+                        long long big_arcs) {
   switch (cluster) {
-    case 2: return desc_launch_cl<2>(table, list, next, smem_deg_max, status, grid, smem, big_arcs, stream);
-    case 4: return desc_launch_cl<4>(table, list, next, smem_deg_max, status, grid, smem, big_arcs, stream);
-    case 8: return desc_launch_cl<8>(table, list, next, smem_deg_max, status, grid, smem, big_arcs, stream);
+    case 2: return desc_launch_cl<2>(table, list, next, smem_deg_max, status, grid, smem, team_arcs, big_arcs, stream);
+    case 4: return desc_launch_cl<4>(table, list, next, smem_deg_max, status, grid, smem, team_arcs, big_arcs, stream);
+    case 8: return desc_launch_cl<8>(table, list, next, smem_deg_max, status, grid, smem, team_arcs, big_arcs, stream);
   }
   cudaError_t e = cudaFuncSetAttribute(desc_peel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  desc_peel<1024><<<grid, 1024, smem, stream>>>(table, list, next, smem_deg_max, status);
+  desc_peel<1024><<<grid, 1024, smem, stream>>>(table, list, next, smem_deg_max, status, team_arcs);
   return cudaGetLastError();
 }
 
-size_t desc_static_smem() { return sizeof(BatchShared<1024>); }
+size_t desc_static_smem() { return sizeof(CtaShared<1024>); }
 
 __global__ void batch_single_gv_kernel(long long* gv, long long n) {
   gv[0] = 0;
@@ -1061,9 +1053,9 @@ int batch_occupancy(int block, size_t smem) {
 
 size_t batch_static_smem(int block) {
   switch (block) {
-    case 256: return sizeof(BatchShared<256>);
-    case 512: return sizeof(BatchShared<512>);
-    case 1024: return sizeof(BatchShared<1024>);
+    case 256: return sizeof(CtaShared<256>);
+    case 512: return sizeof(CtaShared<512>);
+    case 1024: return sizeof(CtaShared<1024>);
   }
   return 0;
 }

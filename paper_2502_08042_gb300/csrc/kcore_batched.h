@@ -60,8 +60,8 @@ struct SlotList {
 // cluster 2, 4 or 8: clusters of that many CTAs for the listed graphs of at
 // least big_arcs arcs (list them largest first)
 cudaError_t desc_launch(const GraphDesc* table, const SlotList& list, int* next, int smem_deg_max,
-                        int* status, int grid, size_t smem, cudaStream_t stream, int cluster = 0,
-                        long long big_arcs = 0);
+                        int* status, int grid, size_t smem, cudaStream_t stream, long long team_arcs,
+                        int cluster = 0, long long big_arcs = 0);
 size_t desc_static_smem();
 // gv = {0, n} on `stream`: the vertex offsets of a batch of one graph
 cudaError_t batch_single_gv(long long* gv, long long n, cudaStream_t stream);

@@ -85,7 +85,7 @@ struct Request {
   int64_t ticket = 0;
   int64_t n = 0, m = 0;
   int32_t* core_h = nullptr;
-  bool large = false;
+  bool large = false, compact = false;
   size_t pool_off = 0, pool_bytes = 0;
   char* d = nullptr;  // device base of the request's pool block
   size_t o_off = 0, o_adj = 0, o_core = 0, o_kmax = 0, o_state = 0;
@@ -102,6 +102,7 @@ struct Batch {
   size_t pool_off = 0, pool_bytes = 0;
   cudaEvent_t done = nullptr;
   int* d_status = nullptr;
+  int stream = 0;  // launch stream
   bool finished = false;
 };
 
@@ -116,7 +117,7 @@ struct kcore_server_ctx {
   PoolAlloc* alloc = nullptr;
   cudaStream_t copy = nullptr, large = nullptr;
   std::vector<cudaStream_t> launch;
-  int next_launch = 0;
+  std::vector<bool> stream_busy;  // a launch is in flight
   std::map<int64_t, Request> reqs;  // by ticket
   std::map<int, Batch> batches;
   int next_batch = 0;
@@ -152,16 +153,18 @@ long long isqrt_s(long long m) {
   return r;
 }
 
-// Whole-GPU peel workspace for a large request (same layout as the handle's).
+// Whole-GPU peel workspace for a large request (same layout as the handle's):
+// for the default schedule, or (compact) without the batch update's counts and
+// with longer slices, for a request that the pool admits only so.
 struct LargeLayout {
-  size_t ctl, rounds, deg, a0, a1, q, total;
+  size_t ctl, rounds, deg, a0, a1, q, hcnt, total;
   long long qcap;
-  int max_rounds;
+  int max_rounds, slice;
 };
-constexpr int kLargeSlice = 64;
-LargeLayout large_layout(long long n, long long m) {
+LargeLayout large_layout(long long n, long long m, bool compact) {
   LargeLayout L{};
-  L.qcap = n + (m + kLargeSlice - 1) / kLargeSlice + 1;
+  L.slice = compact ? 64 : kc::kSliceDefault;
+  L.qcap = n + (m + L.slice - 1) / L.slice + 1;
   L.max_rounds = (int)std::min<long long>(2 * isqrt_s(m) + 8, 2 * n + 8);
   size_t o = 0;
   L.ctl = o;
@@ -176,6 +179,8 @@ LargeLayout large_layout(long long n, long long m) {
   o = al256(o + 4 * (size_t)n);
   L.q = o;
   o = al256(o + 8 * (size_t)L.qcap);
+  L.hcnt = o;
+  if (!compact) o = al256(o + 4 * (size_t)n);
   L.total = o;
   return L;
 }
@@ -248,6 +253,7 @@ kcore_status kcore_server_create(kcore_server* out, int device, const kcore_serv
   cudaStreamCreateWithFlags(&s->copy, cudaStreamNonBlocking);
   cudaStreamCreateWithFlags(&s->large, cudaStreamNonBlocking);
   s->launch.resize(c.streams);
+  s->stream_busy.assign(c.streams, false);
   for (auto& st : s->launch) cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
   if (cudaHostAlloc((void**)&s->pinned, sizeof(int32_t) * 2 * (size_t)c.max_requests, cudaHostAllocDefault) !=
       cudaSuccess) {
@@ -301,10 +307,14 @@ kcore_status kcore_server_submit(kcore_server s, int64_t n, int64_t m, const int
   r.o_kmax = o;
   o = al256(o + 8);
   r.o_state = o;
-  if (r.large) o += large_layout(n, m).total;
+  if (r.large) o += large_layout(n, m, false).total;
   else o += 5 * al256(4 * (size_t)std::max<int64_t>(n, 1));
   size_t poff = 0;
-  if (!s->alloc->alloc(o, &poff)) return KCORE_ERR_CAPACITY;  // not admitted now
+  if (!s->alloc->alloc(o, &poff)) {
+    r.compact = r.large;
+    if (r.compact) o = r.o_state + large_layout(n, m, true).total;
+    if (!r.compact || !s->alloc->alloc(o, &poff)) return KCORE_ERR_CAPACITY;  // not admitted now
+  }
   r.pool_off = poff;
   r.pool_bytes = o;
   r.d = s->pool + poff;
@@ -369,8 +379,14 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
     if (r.state == RS_READY && !r.large) small_ready.push_back(r.ticket);
   }
   cudaGetLastError();  // cudaEventQuery's cudaErrorNotReady is not an error
-  // 2a. batched launches for the small requests that became ready together
+  // 2a. batched launches for the small requests that became ready together,
+  // one in flight per launch stream: behind a running launch the requests
+  // would wait all the same, and those that gather meanwhile make one launch
+  // that fills the GPU instead of a queue of launches of a few graphs each.
   for (size_t first = 0; first < small_ready.size(); first += kc::kMaxSlotsPerLaunch) {
+    size_t idle = 0;
+    while (idle < s->launch.size() && s->stream_busy[idle]) idle++;
+    if (idle == s->launch.size()) break;
     int cnt = (int)std::min<size_t>(small_ready.size() - first, (size_t)kc::kMaxSlotsPerLaunch);
     Batch b;
     if (!s->alloc->alloc(256, &b.pool_off)) break;  // no room for the counters now: next poll
@@ -395,8 +411,7 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
       r.batch = s->next_batch;
       b.reqs.push_back(r.ticket);
     }
-    cudaStream_t st = s->launch[s->next_launch];
-    s->next_launch = (s->next_launch + 1) % (int)s->launch.size();
+    cudaStream_t st = s->launch[idle];
     const int cl = s->cfg.batch_cluster > 1 ? s->cfg.batch_cluster : 0;
     int grid = std::min(cl ? cnt * cl : cnt, s->desc_grid_cap);
     long long big = s->cfg.batch_big_arcs > 0 ? (long long)s->cfg.batch_big_arcs
@@ -404,7 +419,8 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
     e = cudaMemsetAsync(ctr, 0, 2 * sizeof(int), st);
     if (e == cudaSuccess)
       e = kc::desc_launch(s->d_table, list, ctr, (int)s->smem_vertices, b.d_status, grid,
-                          s->smem_vertices * 4, st, cl, big);
+                          s->smem_vertices * 4, st, std::max<long long>(1, launch_arcs / std::max(grid, 1) / 2), cl,
+                          big);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventRecord(b.done, st);
     if (e != cudaSuccess) {
@@ -412,13 +428,15 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
       s->err = std::string("batched launch: ") + cudaGetErrorString(e);
       return KCORE_ERR_CUDA;
     }
+    b.stream = (int)idle;
+    s->stream_busy[idle] = true;
     s->batches.emplace(s->next_batch++, b);
   }
   // 2b. large requests: the whole-GPU single-graph peel, one at a time on its stream
   for (auto& kv : s->reqs) {
     Request& r = kv.second;
     if (r.state != RS_READY || !r.large) continue;
-    LargeLayout L = large_layout(r.n, r.m);
+    LargeLayout L = large_layout(r.n, r.m, r.compact);
     char* ws = r.d + r.o_state;
     kc::PeelArgs a{};
     a.n = r.n;
@@ -435,20 +453,24 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
     a.rounds = (kc::RoundRec*)(ws + L.rounds);
     a.max_rounds = L.max_rounds;
     a.ctl = (kc::PeelCtl*)(ws + L.ctl);
-    a.slice = kLargeSlice;
-    a.lq_cap = 32;
+    // the handle's default schedule
+    a.slice = L.slice;
+    a.lq_cap = kc::kLocalQueueDefault;
     a.max_take = 256;
-    a.scan_min = 2048;
+    a.scan_min = kc::kScanMin;
     a.idle_sleep_ns = 192;
-    a.poll_sleep_ns = 64;
+    a.poll_sleep_ns = kc::kPollSleepDefault;
     a.timeout_ns = 2000ull * 1000000ull;
     long long want = (r.n + r.m / 8 + 2047) / 2048;
     long long gmax = (long long)s->sms * s->peel_ctas_per_sm;
     int grid = (int)std::max<long long>(1, std::min(want, gmax));
     a.take_div = grid * (kc::bsp_block_size() / 32);
-    a.local_batches = 8;
-    a.precheck_items = 64;
+    a.local_batches = kc::kLocalBatchesDefault;
+    a.precheck_items = kc::kPrecheckDefault;
+    a.hybrid = r.compact ? 0 : 1;
+    a.hcnt = (int*)(ws + L.hcnt);
     e = cudaMemsetAsync(ws, 0, L.deg, s->large);
+    if (e == cudaSuccess && a.hybrid) e = cudaMemsetAsync(a.hcnt, 0, 4 * (size_t)r.n, s->large);
     if (e == cudaSuccess) e = kc::bsp_launch(a, grid, s->large);
     if (e == cudaSuccess) e = cudaEventRecord(r.ev, s->large);
     if (e != cudaSuccess) {
@@ -464,6 +486,7 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
     Batch& b = kv.second;
     if (b.finished || cudaEventQuery(b.done) != cudaSuccess) continue;
     b.finished = true;
+    s->stream_busy[b.stream] = false;
     for (int64_t t : b.reqs) {
       Request& r = s->reqs[t];
       if (r.n > 0) cudaMemcpyAsync(r.core_h, r.d + r.o_core, 4 * (size_t)r.n, cudaMemcpyDeviceToHost, s->copy);
@@ -476,7 +499,7 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
   for (auto& kv : s->reqs) {
     Request& r = kv.second;
     if (r.state != RS_RUNNING || !r.large || cudaEventQuery(r.ev) != cudaSuccess) continue;
-    LargeLayout L = large_layout(r.n, r.m);
+    LargeLayout L = large_layout(r.n, r.m, r.compact);
     char* ws = r.d + r.o_state;
     if (r.n > 0) cudaMemcpyAsync(r.core_h, r.d + r.o_core, 4 * (size_t)r.n, cudaMemcpyDeviceToHost, s->copy);
     cudaMemcpyAsync(r.kmax_slot, r.d + r.o_kmax, 4, cudaMemcpyDeviceToHost, s->copy);
