@@ -161,36 +161,27 @@ __device__ __forceinline__ unsigned long long make_item(long long a0, long long 
 }
 
 // Writes each lane's arc range [e0, e1), cut in `cnt` slices, to the queue:
-// the warp's tot slices go to p0 on, this lane's after excl of them. Lanes with
-// a slice or two each write their own; else the slices are spread over the
-// warp (a slice's lane by a search over the lanes' excl), so a hub's are not
-// stored by one lane and the stores are consecutive. Warp-collective.
+// the warp's tot slices go to p0 on, this lane's after excl of them. A lane
+// writes up to kOwn slices itself; a longer range's (a hub's, or any list at a
+// high level) are written by the whole warp with consecutive stores.
+// Warp-collective.
 __device__ __forceinline__ void write_slices(const PeelArgs& a, long long e0, long long e1, int cnt,
                                              unsigned long long p0, int excl, int tot, int lane) {
+  constexpr int kOwn = 8;
   const bool pf = tot <= kPrefetchSlices;
-  if (!__any_sync(kFull, cnt > 2)) {
-    if (cnt > 0) {
-      a.Q[p0 + excl] = make_item(e0, min((long long)a.slice, e1 - e0));
-      if (pf) prefetch_arcs(a, e0);
-    }
-    if (cnt > 1) {
-      a.Q[p0 + excl + 1] = make_item(e0 + a.slice, e1 - e0 - a.slice);
-      if (pf) prefetch_arcs(a, e0 + a.slice);
-    }
-    return;
-  }
-  for (int j0 = 0; j0 < tot; j0 += kWarp) {
-    const int j = j0 + lane;
-    int L = 0;  // the last lane with excl <= j holds slice j
-#pragma unroll
-    for (int s = kWarp / 2; s > 0; s >>= 1)
-      if (__shfl_sync(kFull, excl, L + s) <= j) L += s;
+  auto write = [&](unsigned long long p, long long b0, long long b1, int i) {
+    const long long s0 = b0 + (long long)i * a.slice;
+    a.Q[p + i] = make_item(s0, min((long long)a.slice, b1 - s0));
+    if (pf) prefetch_arcs(a, s0);
+  };
+  if (cnt <= kOwn)
+    for (int i = 0; i < cnt; i++) write(p0 + excl, e0, e1, i);
+  for (unsigned big = __ballot_sync(kFull, cnt > kOwn); big; big &= big - 1) {
+    const int L = __ffs(big) - 1;
     const long long b0 = __shfl_sync(kFull, e0, L), b1 = __shfl_sync(kFull, e1, L);
-    const long long s0 = b0 + (long long)(j - __shfl_sync(kFull, excl, L)) * a.slice;
-    if (j < tot) {
-      a.Q[p0 + j] = make_item(s0, min((long long)a.slice, b1 - s0));
-      if (pf) prefetch_arcs(a, s0);
-    }
+    const int bc = __shfl_sync(kFull, cnt, L);
+    const unsigned long long bp = p0 + __shfl_sync(kFull, excl, L);
+    for (int i = lane; i < bc; i += kWarp) write(bp, b0, b1, i);
   }
 }
 
