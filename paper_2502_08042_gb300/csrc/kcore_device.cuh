@@ -34,6 +34,15 @@ __device__ __forceinline__ int ld_acquire_s32(const int* p) {
   asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
+// A kernel launched with programmatic stream serialisation starts while its
+// predecessor drains: it lets its own successor start and then waits here
+// until the predecessor is complete and its writes are visible. First
+// statement of every kernel launched so.
+__device__ __forceinline__ void wait_predecessor() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Streaming read of data used once (adjacency): do not keep it in L1, mark it
 // evict-first in L2 so the induced-degree array stays resident.
 __device__ __forceinline__ int ld_stream_s32(const int* p) { return __ldcs(p); }
