@@ -51,6 +51,7 @@ namespace kc {
 template <int BLOCK>
 constexpr int kBatchIlp = BLOCK >= 1024 ? 8 : 4;
 constexpr int kScanItems = 8;  // active-list entries per thread per scan tile
+constexpr int kPackShare = 8;  // the active list is rewritten when 1 / kPackShare of it is peeled
 
 template <int BLOCK>
 struct BatchShared {
@@ -355,16 +356,18 @@ __device__ __forceinline__ int tile_entry(int q) {
 }
 
 // The kept (d >= keep_from) and taken (d == take_at) entries of a tile, packed
-// taken << 16 | kept: *total for the tile; returns those ahead of this warp.
+// taken << 16 | kept: *total for the tile, *own for this warp; returns those
+// ahead of it.
 template <int BLOCK>
 __device__ __forceinline__ int tile_count(const int (&d)[kScanItems], int keep_from, int take_at,
-                                          BatchShared<BLOCK>& sh, int& ph, int* total) {
+                                          BatchShared<BLOCK>& sh, int& ph, int* total, int* own) {
   constexpr int kW = BLOCK / 32;
   const int lane = threadIdx.x & 31, warp = team_tid<BLOCK>() >> 5;
   int sum = 0;
 #pragma unroll
   for (int q = 0; q < kScanItems; q++) sum += (d[q] >= keep_from ? 1 : 0) + (d[q] == take_at ? 1 << 16 : 0);
   sum = (int)__reduce_add_sync(kFull, (unsigned)sum);
+  *own = sum;
   int* part = sh.part[ph];
   ph ^= 1;
   if (lane == 0) part[warp] = sum;
@@ -388,7 +391,8 @@ __device__ __forceinline__ void tile_write(const int (&v)[kScanItems], const int
 }
 
 // One pass over the active list after level k: entries with D > k survive
-// into `out` (their minimum goes to *dmin); among them, those at exactly k+1
+// into `out` (nullptr: the list stays as it is; their minimum goes to *dmin);
+// among them, those at exactly k+1
 // are also written to F (the next frontier if level k+1 is not empty).
 // Returns the survivors; *nf gets the number written to F.
 template <int BLOCK>
@@ -411,10 +415,10 @@ __device__ int compact_active(const int* A, int la, int n, int* out, int* F, con
 #pragma unroll
     for (int q = 0; q < kScanItems; q++)
       if (d[q] > k) lmin = min(lmin, d[q]);  // (no entry: -1)
-    int tot;
-    const int at = tile_count(d, k + 1, k + 1, sh, ph, &tot);
-    tile_write(v, d, out + written + (at & 0xffff), [k](int x) { return x > k; });
-    tile_write(v, d, F + wf + (at >> 16), [k](int x) { return x == k + 1; });
+    int tot, own;
+    const int at = tile_count(d, k + 1, k + 1, sh, ph, &tot, &own);
+    if (out) tile_write(v, d, out + written + (at & 0xffff), [k](int x) { return x > k; });
+    if (own >> 16) tile_write(v, d, F + wf + (at >> 16), [k](int x) { return x == k + 1; });
     written += tot & 0xffff;
     wf += tot >> 16;
   }
@@ -443,9 +447,9 @@ __device__ int select_frontier(const int* A, int la, int n, int* F, const DegSto
     }
     int d[kScanItems];
     D.get_all(v, d);
-    int tot;
-    const int at = tile_count(d, INT_MAX, k, sh, ph, &tot);
-    tile_write(v, d, F + written + (at >> 16), [k](int x) { return x == k; });
+    int tot, own;
+    const int at = tile_count(d, INT_MAX, k, sh, ph, &tot, &own);
+    if (own) tile_write(v, d, F + written + (at >> 16), [k](int x) { return x == k; });
     written += tot >> 16;
   }
   team_sync<BLOCK>();  // the frontier is read by other threads next
@@ -506,6 +510,7 @@ __device__ void peel_one_graph(int smem_deg_max, int* status, int* sdeg, BatchSh
   for (int v = tid; v < n; v += BLOCK) __stcs(gd.A0 + v, v);
   team_sync<BLOCK>();
   bool odd = false;  // the active list is in A1
+  int peeled = 0;    // its entries peeled since it was written
   int la = n;
   int kmax = 0;
   int r = 0;  // subrounds: frontier counter r & 1 counts this one's appends
@@ -513,6 +518,7 @@ __device__ void peel_one_graph(int smem_deg_max, int* status, int* sdeg, BatchSh
   for (;;) {
     bool fodd = false;  // the frontier is in F1
     while (nf > 0) {
+      peeled += nf;
       for (int c0 = 0; c0 < nf; c0 += BLOCK) {
         const int cnum = min(BLOCK, nf - c0);
         const int total = load_chunk<BLOCK>(gd, (fodd ? gd.F1 : gd.F0) + c0, cnum, n, k, true, status, sh, ph);
@@ -527,13 +533,21 @@ __device__ void peel_one_graph(int smem_deg_max, int* status, int* sdeg, BatchSh
       fodd = !fodd;
     }
     kmax = k;
-    // drop the vertices peeled at level k; the minimum induced degree of the
-    // rest is the next non-empty level; vertices at k+1 are collected on the
-    // way in case that level is the next one
+    // The minimum induced degree of the vertices left is the next non-empty
+    // level; vertices at k+1 are collected on the way in case that level is
+    // the next one. The list is rewritten without the peeled vertices once
+    // they are kPackShare of it: a deep graph's levels peel a percent or two
+    // each, and the stores are a third of a tile's time.
+    const bool pack = (long long)peeled * kPackShare >= la;
     int dmin;
-    la = compact_active<BLOCK>(odd ? gd.A1 : gd.A0, la, n, odd ? gd.A0 : gd.A1, gd.F0, D, k, sh, ph, &dmin, &nf);
-    odd = !odd;
-    if (la == 0) break;
+    const int left = compact_active<BLOCK>(odd ? gd.A1 : gd.A0, la, n, pack ? (odd ? gd.A0 : gd.A1) : nullptr, gd.F0, D, k,
+                                           sh, ph, &dmin, &nf);
+    if (left == 0) break;
+    if (pack) {
+      la = left;
+      odd = !odd;
+      peeled = 0;
+    }
     if (dmin != k + 1) nf = select_frontier<BLOCK>(odd ? gd.A1 : gd.A0, la, n, gd.F0, D, dmin, sh, ph);
     k = dmin;
   }
@@ -607,11 +621,11 @@ struct ClusterPeel {
       }
       int d[kScanItems];
       D.get_all(v, d);
-      int tot;
-      const int at = tile_count(d, INT_MAX, k, sh, sp, &tot);
+      int tot, own;
+      const int at = tile_count(d, INT_MAX, k, sh, sp, &tot, &own);
       if (threadIdx.x == 0) sh.base = tot ? atomicAdd(&slot(ph)[0], tot >> 16) : 0;
       __syncthreads();
-      tile_write(v, d, F + sh.base + (at >> 16), [k](int x) { return x == k; });
+      if (own) tile_write(v, d, F + sh.base + (at >> 16), [k](int x) { return x == k; });
       __syncthreads();  // sh.base is reused by the next tile
     }
   }
@@ -637,8 +651,8 @@ struct ClusterPeel {
 #pragma unroll
       for (int q = 0; q < kScanItems; q++)
         if (d[q] > k) lmin = min(lmin, d[q]);  // (no entry: -1)
-      int tot;
-      const int at = tile_count(d, k + 1, k + 1, sh, sp, &tot);
+      int tot, own;
+      const int at = tile_count(d, k + 1, k + 1, sh, sp, &tot, &own);
       if (threadIdx.x == 0) {
         const int bk = (tot & 0xffff) ? atomicAdd(&slot(ph)[0], tot & 0xffff) : 0;
         const int bf = (tot >> 16) ? atomicAdd(&slot(ph)[1], tot >> 16) : 0;
@@ -647,7 +661,7 @@ struct ClusterPeel {
       }
       __syncthreads();
       tile_write(v, d, out + sh.base + (at & 0xffff), [k](int x) { return x > k; });
-      tile_write(v, d, F + sh.base2 + (at >> 16), [k](int x) { return x == k + 1; });
+      if (own >> 16) tile_write(v, d, F + sh.base2 + (at >> 16), [k](int x) { return x == k + 1; });
       __syncthreads();
     }
     int none = INT_MAX;
