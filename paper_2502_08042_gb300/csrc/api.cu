@@ -403,8 +403,10 @@ kcore_status peel_call(kcore_ctx* h, int64_t n, int64_t m, const int64_t* offset
   const int mode = threshold ? 2 : effective_mode(h);
   const int slice =
       h->opt[KCORE_OPT_SLICE_ARCS] > 0 ? (int)h->opt[KCORE_OPT_SLICE_ARCS] : (mode == 1 ? 512 : kc::kSliceDefault);
+  // (a k'-core query of a small graph or a small k' has no pass heavy enough for
+  // the batch update: clearing its counts would add 5 us to some 65)
   bool hybrid = mode == 2 && h->opt[KCORE_OPT_BATCH_UPDATE] != 0 &&
-                (threshold || h->opt[KCORE_OPT_LEVEL_WINDOW] == 0);
+                (threshold ? m >= ((int64_t)1 << 22) && kprime >= 16 : h->opt[KCORE_OPT_LEVEL_WINDOW] == 0);
   const bool sample = sampling_on(h, threshold);
   PeelLayout L = peel_layout(n, m, slice, mode == 3 || hybrid, sample);
   if (threshold && h->ws_external && h->ws_bytes < L.total) {

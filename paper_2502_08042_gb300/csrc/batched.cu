@@ -89,8 +89,19 @@ __device__ __forceinline__ void flag_bad(int* status, int code, long long value,
   *bad = 1;
 }
 
+// The sum of the first `warp` of the kW warps' values, and their total. By two
+// warp reductions: every warp of the CTA runs this, and a scan's shuffles (one
+// warp instruction per cycle and SM) cost more than the barrier it replaces.
+template <int kW>
+__device__ __forceinline__ int warps_ahead(const int* part, int* total) {
+  const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) & (kW - 1);
+  const unsigned p = lane < kW ? (unsigned)part[lane] : 0u;
+  *total = (int)__reduce_add_sync(kFull, p);
+  return (int)__reduce_add_sync(kFull, lane < warp ? p : 0u);
+}
+
 // Block-wide exclusive scan of one int per thread; returns the exclusive value,
-// *total gets the sum. One barrier: every warp scans the warps' sums itself,
+// *total gets the sum. One barrier: every warp sums the warps' sums itself,
 // and the sums alternate between two arrays (ph, toggled here), so the next
 // scan's stores cannot meet this one's loads.
 template <int BLOCK>
@@ -102,10 +113,7 @@ __device__ __forceinline__ int block_excl_scan(int x, BatchShared<BLOCK>& sh, in
   ph ^= 1;
   if (lane == 31) part[warp] = incl;
   team_sync<BLOCK>();
-  const int p = lane < kW ? part[lane] : 0;
-  const int pi = warp_incl_scan(p, lane);
-  *total = __shfl_sync(kFull, pi, kW - 1);
-  return __shfl_sync(kFull, pi - p, warp) + incl - x;
+  return warps_ahead<kW>(part, total) + incl - x;
 }
 
 // Block-wide minimum of two values (one barrier; the callers have another
@@ -114,15 +122,15 @@ template <int BLOCK>
 __device__ __forceinline__ void block_min2(int& x, int& y, BatchShared<BLOCK>& sh) {
   constexpr int kW = BLOCK / 32;
   const int lane = threadIdx.x & 31, warp = team_tid<BLOCK>() >> 5;
-  x = warp_min(x);
-  y = warp_min(y);
+  x = __reduce_min_sync(kFull, x);
+  y = __reduce_min_sync(kFull, y);
   if (lane == 0) {
     sh.red[0][warp] = x;
     sh.red[1][warp] = y;
   }
   team_sync<BLOCK>();
-  x = warp_min(lane < kW ? sh.red[0][lane] : INT_MAX);
-  y = warp_min(lane < kW ? sh.red[1][lane] : INT_MAX);
+  x = __reduce_min_sync(kFull, lane < kW ? sh.red[0][lane] : INT_MAX);
+  y = __reduce_min_sync(kFull, lane < kW ? sh.red[1][lane] : INT_MAX);
 }
 
 // The induced degrees d~ of one graph, in shared memory or in L2 (atomics are
@@ -256,10 +264,10 @@ __device__ __forceinline__ int load_chunk(const GraphDesc& gd, const int* F, int
 // makes each wait for the one before), and the crossing vertices of kBatchIlp
 // windows are appended to Fn with one atomic. Every list of a chunk holds an
 // arc: a frontier vertex of level k >= 1 has degree >= k.
-template <int BLOCK, int kMode, bool kNarrow>
+template <int BLOCK, int kIlp, int kMode, bool kNarrow>
 __device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& D, int n, int k, int jlo, int jhi,
                                            int cnum, int* Fn, int* counter, int* status, BatchShared<BLOCK>& sh) {
-  constexpr int kW = BLOCK / 32, kIlp = kBatchIlp<BLOCK>;
+  constexpr int kW = BLOCK / 32;
   const int lane = threadIdx.x & 31, warp = team_tid<BLOCK>() >> 5;
   const int run = ((((jhi - jlo + 31) >> 5) + kW - 1) / kW) << 5;  // arcs per warp
   int j0 = jlo + warp * run;
@@ -336,24 +344,42 @@ __device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& 
 template <int BLOCK>
 __device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& D, int n, int k, int jlo, int jhi,
                                            int cnum, int* Fn, int* counter, int* status, BatchShared<BLOCK>& sh) {
-#define KC_ARCS(MODE)                                                                                            \
-  (D.narrow ? chunk_arcs<BLOCK, MODE, true>(gd, D, n, k, jlo, jhi, cnum, Fn, counter, status, sh)                  \
-            : chunk_arcs<BLOCK, MODE, false>(gd, D, n, k, jlo, jhi, cnum, Fn, counter, status, sh))
+  // at most one window per warp: without the slots of further windows, whose
+  // instructions alone would be most of a small graph's phase
+#define KC_ARCS2(ILP, MODE)                                                                                     \
+  (D.narrow ? chunk_arcs<BLOCK, ILP, MODE, true>(gd, D, n, k, jlo, jhi, cnum, Fn, counter, status, sh)             \
+            : chunk_arcs<BLOCK, ILP, MODE, false>(gd, D, n, k, jlo, jhi, cnum, Fn, counter, status, sh))
+#define KC_ARCS(MODE)                           \
+  do {                                          \
+    if (jhi - jlo <= BLOCK) KC_ARCS2(1, MODE);  \
+    else KC_ARCS2(kBatchIlp<BLOCK>, MODE);      \
+  } while (0)
   if (D.mode == kDegSmem) KC_ARCS(kDegSmem);
   else if (D.mode == kDegGlobal) KC_ARCS(kDegGlobal);
   else KC_ARCS(kDegSplit);
+#undef KC_ARCS2
 #undef KC_ARCS
 }
 
-// Entry q of this thread in a tile of BLOCK * kScanItems list entries: a warp
-// takes consecutive entries, 32 per q, so its loads and the stores of what it
-// keeps are consecutive. (Eight entries per thread side by side in the output
-// put every lane of a store in a sector of its own: 4,700 of a tile's 10,700
-// cycles.)
-template <int BLOCK>
-__device__ __forceinline__ int tile_entry(int q) {
-  return (team_tid<BLOCK>() >> 5) * (32 * kScanItems) + q * 32 + (int)(threadIdx.x & 31);
-}
+// A tile of BLOCK * kScanItems list entries: a warp takes consecutive entries,
+// 32 per slot, so its loads and the stores of what it keeps are consecutive.
+// (Eight entries per thread side by side in the output put every lane of a
+// store in a sector of its own: 4,700 of a tile's 10,700 cycles.) A short tile
+// fills fewer slots, not fewer warps.
+struct TileMap {
+  int first, end, rows;  // this thread's first entry, the tile's end, the slots filled
+  template <int BLOCK>
+  __device__ __forceinline__ static TileMap at(int base, int len) {
+    const int rows = min(kScanItems, (len - base + BLOCK - 1) / BLOCK);
+    return TileMap{base + (team_tid<BLOCK>() >> 5) * (32 * rows) + (int)(threadIdx.x & 31), min(len, base + BLOCK * rows),
+                   rows};
+  }
+  // the list index of slot q, or -1
+  __device__ __forceinline__ int entry(int q) const {
+    const int i = first + q * 32;
+    return q < rows && i < end ? i : -1;
+  }
+};
 
 // The kept (d >= keep_from) and taken (d == take_at) entries of a tile, packed
 // taken << 16 | kept: *total for the tile, *own for this warp; returns those
@@ -372,10 +398,7 @@ __device__ __forceinline__ int tile_count(const int (&d)[kScanItems], int keep_f
   ph ^= 1;
   if (lane == 0) part[warp] = sum;
   team_sync<BLOCK>();
-  const int p = lane < kW ? part[lane] : 0;
-  const int pi = warp_incl_scan(p, lane);
-  *total = __shfl_sync(kFull, pi, kW - 1);
-  return __shfl_sync(kFull, pi - p, warp);
+  return warps_ahead<kW>(part, total);
 }
 
 // Writes the entries v[q] of the lanes with want(d[q]) to out, in list order.
@@ -400,12 +423,13 @@ __device__ int compact_active(const int* A, int la, int n, int* out, int* F, con
                               BatchShared<BLOCK>& sh, int& ph, int* dmin, int* nf) {
   int written = 0, wf = 0, lmin = INT_MAX;
   for (int base = 0; base < la; base += BLOCK * kScanItems) {
+    const TileMap tm = TileMap::at<BLOCK>(base, la);
     int v[kScanItems];
 #pragma unroll
     for (int q = 0; q < kScanItems; q++) {
-      int i = base + tile_entry<BLOCK>(q);
+      const int i = tm.entry(q);
       v[q] = -1;
-      if (i < la) {
+      if (i >= 0) {
         int x = __ldcs(A + i);
         v[q] = (unsigned)x < (unsigned)n ? x : -1;  // ids are < n by construction; checked anyway
       }
@@ -435,12 +459,13 @@ __device__ int select_frontier(const int* A, int la, int n, int* F, const DegSto
                                BatchShared<BLOCK>& sh, int& ph) {
   int written = 0;
   for (int base = 0; base < la; base += BLOCK * kScanItems) {
+    const TileMap tm = TileMap::at<BLOCK>(base, la);
     int v[kScanItems];
 #pragma unroll
     for (int q = 0; q < kScanItems; q++) {
-      int i = base + tile_entry<BLOCK>(q);
+      const int i = tm.entry(q);
       v[q] = -1;
-      if (i < la) {
+      if (i >= 0) {
         int x = __ldcs(A + i);
         v[q] = (unsigned)x < (unsigned)n ? x : -1;  // ids are < n by construction; checked anyway
       }
@@ -609,12 +634,13 @@ struct ClusterPeel {
   __device__ void select(const int* A, int la, int n, int* F, const DegStore& D, int k) {
     const int lo = (int)part_lo(la), hi = (int)part_hi(la);
     for (int base = lo; base < hi; base += BLOCK * kScanItems) {
+      const TileMap tm = TileMap::at<BLOCK>(base, hi);
       int v[kScanItems];
 #pragma unroll
       for (int q = 0; q < kScanItems; q++) {
-        const int i = base + tile_entry<BLOCK>(q);
+        const int i = tm.entry(q);
         v[q] = -1;
-        if (i < hi) {
+        if (i >= 0) {
           const int x = __ldcg(A + i);  // written by other CTAs of the cluster
           v[q] = (unsigned)x < (unsigned)n ? x : -1;
         }
@@ -636,12 +662,13 @@ struct ClusterPeel {
     const int lo = (int)part_lo(la), hi = (int)part_hi(la);
     int lmin = INT_MAX;
     for (int base = lo; base < hi; base += BLOCK * kScanItems) {
+      const TileMap tm = TileMap::at<BLOCK>(base, hi);
       int v[kScanItems];
 #pragma unroll
       for (int q = 0; q < kScanItems; q++) {
-        const int i = base + tile_entry<BLOCK>(q);
+        const int i = tm.entry(q);
         v[q] = -1;
-        if (i < hi) {
+        if (i >= 0) {
           const int x = __ldcg(A + i);
           v[q] = (unsigned)x < (unsigned)n ? x : -1;
         }
