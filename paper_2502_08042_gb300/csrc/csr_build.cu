@@ -11,17 +11,16 @@
 //      digits. Each CTA owns a contiguous chunk; a pass is an upsweep (digit
 //      histogram per CTA), a scan of each digit's row of the 256 x CTAs
 //      histogram (one CTA per digit), and a downsweep that ranks each
-//      2,048-key tile in shared memory and writes runs of equal digits
-//      contiguously, while the next tile arrives by asynchronous copy
-//      (cp.async). A key's rank within its warp and digit comes from one pass:
-//      the lanes holding a digit elect a leader (warp match), which adds their
-//      number to the warp's counter for that digit and hands the old value on.
+//      4,096-key tile in shared memory and writes runs of equal digits
+//      contiguously, while the next tile's lines are prefetched. A key's rank
+//      within its warp and digit comes from one pass over the warp's rows: the
+//      lanes holding a digit or their bits into the warp's counter for it.
 //   3. unique + emit: keys equal to their predecessor are dropped; the rest
 //      are written in order as adj[] (low B bits), and the first arc of each
 //      source vertex fixes offsets[] (vertices without arcs take the next
-//      vertex's offset). Keys are read striped (a warp reads 32 consecutive
-//      keys), the predecessor comes from the next lower lane, and the
-//      positions from warp ballots, so no key passes through shared memory.
+//      vertex's offset). Each warp walks a chunk of its own in rows of 32 keys;
+//      the predecessor comes from the next lower lane or row and the positions
+//      from warp ballots, so no key passes through shared memory.
 // A single graph, and a batch for which it means fewer keys to move, takes the
 // edge route through steps 1-3: each pair (a, b) with a != b gives ONE key
 // (min << B) | max (global ids); sorting these E keys by both
@@ -250,9 +249,9 @@ __global__ void __launch_bounds__(1024) scan_u32_to_u64(const unsigned* in, unsi
 // order. offs[d * G + g] counts the keys of digit d in the chunks before g,
 // rowtot[d] all keys of digit d; so the CTA's first key of digit d goes after
 // every key of a smaller digit and the digit-d keys of earlier chunks.
-// kArcs / kCanon: the first pass, whose keys are made from the edge list (a
-// tile is 1,024 edges / 2,048 edges; the order within a tile does not matter
-// in the first pass).
+// kArcs / kCanon / kCanonB: the first pass, whose keys are made from the edge
+// list (a tile is 2,048 edges / 4,096 edges; the order within a tile does not
+// matter in the first pass).
 // Pos: the type of an output position (32 bits when there are at most 2^32
 // keys: positions are then computed modulo 2^32).
 static_assert(kCsrBlock == 256, "one thread per 8-bit digit");
