@@ -878,7 +878,9 @@ __device__ long long peel_drawn(const Source& src, int smem_deg_max, int* sdeg, 
     if (gi >= src.count()) return -1;
     Found f;
     if (!src.find(gi, tid == 0, &sh.bad, &f)) continue;
-    if (f.arcs < stop_below) return gi;
+    // (0: never. A malformed graph may count fewer than no arcs: it is peeled
+    // here all the same, so that peel_one_graph's checks report it)
+    if (stop_below > 0 && f.arcs < stop_below) return gi;
     if (tid == 0) sh.gd = src.desc(f);
     team_sync<BLOCK>();
     peel_one_graph<BLOCK>(smem_deg_max, src.status(), sdeg, sh);
