@@ -25,6 +25,7 @@
 
 #include "kcore_device.cuh"
 #include "kcore_peel.h"
+#include "kcore_search.h"
 
 namespace kc {
 
@@ -159,11 +160,11 @@ __global__ void __launch_bounds__(256) csr_validate_arcs(long long n, long long 
         int y[kRows];
 #pragma unroll
         for (int q = 0; q < kRows; q++)
-          y[q] = ((left >> q) & 1u) && lo[q] < hi[q] ? adj[o0[q] + ((lo[q] + hi[q]) >> 1)] : 0;
+          y[q] = ((left >> q) & 1u) && lo[q] < hi[q] ? adj[o0[q] + middle(lo[q], hi[q])] : 0;
 #pragma unroll
         for (int q = 0; q < kRows; q++) {
           if (!((left >> q) & 1u)) continue;
-          const int mid = (lo[q] + hi[q]) >> 1;
+          const int mid = middle(lo[q], hi[q]);
           if (lo[q] >= hi[q]) record(st, 6, v[q], row + q * 32 + lane);
           if (lo[q] >= hi[q] || y[q] == v[q]) left &= ~(1u << q);
           else if (y[q] < v[q]) lo[q] = mid + 1;

@@ -45,3 +45,19 @@ def test_rows(gap, hub):
                 assert e.value.code == "NOT_SIMPLE"
                 st = k.stats()
                 assert (st["invalid_check"], st["invalid_vertex"]) == (6, int(adj[j]))
+
+
+def test_hub_of_more_than_2_to_30_arcs():
+    """A star of 2^30 + 1,000 leaves, its hub without the arc to the last leaf:
+    the third launch searches every leaf's arc in the hub's list."""
+    leaves = (1 << 30) + 1000
+    adj = torch.zeros(2 * leaves - 1, dtype=torch.int32, device="cuda")
+    adj[:leaves - 1] = torch.arange(1, leaves, dtype=torch.int32, device="cuda")
+    off = torch.arange(leaves - 2, 2 * leaves, dtype=torch.int64, device="cuda")
+    off[0] = 0
+    with KCore(0) as k:
+        with pytest.raises(KCoreError) as e:
+            k.validate_csr(off, adj)
+        assert e.value.code == "NOT_SIMPLE"
+        s = k.stats()
+        assert (s["invalid_check"], s["invalid_vertex"], s["invalid_arc"]) == (6, leaves, 2 * leaves - 2)
