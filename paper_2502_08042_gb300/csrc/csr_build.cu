@@ -433,7 +433,7 @@ struct WarpKeys {
       const long long i = ts + q * 32 + lane;
       x[q] = i < hi ? __ldcs(k + i) : kSentinel;
     }
-    next = ts + kUTile < N ? __ldg(k + ts + kUTile) : kSentinel;
+    next = ts + kUTile < N ? k[ts + kUTile] : kSentinel;
   }
   __device__ __forceinline__ unsigned long long pred(int q, int lane) const {
     const unsigned long long up = __shfl_up_sync(kFull, x[q], 1);
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(kCsrBlock) csr_count_unique(const unsigned lon
   const long long lo = w * chunk, hi = min(N, lo + chunk);
   unsigned c = 0;
   WarpKeys t;
-  t.prev = lo > 0 && lo < hi ? __ldg(k + lo - 1) : kSentinel;
+  t.prev = lo > 0 && lo < hi ? k[lo - 1] : kSentinel;
   for (long long ts = lo; ts < hi; ts += kUTile) {
     t.load(k, ts, hi, N, lane);
 #pragma unroll
@@ -506,14 +506,10 @@ __global__ void __launch_bounds__(kCsrBlock) csr_count_unique(const unsigned lon
 //     starts[x]); m = twice A's unique keys. gv: a batch's ids leave graph-local.
 enum EmitMode : int { kEmitAll = 0, kEmitUpper = 2 };
 template <int kMode>
-__global__ void __launch_bounds__(kCsrBlock) csr_emit(const unsigned long long* __restrict__ k, long long N,
-                                                      long long chunk, int B, long long n,
-                                                      const unsigned long long* __restrict__ base,
-                                                      int* __restrict__ adj, long long* __restrict__ off,
-                                                      long long* __restrict__ m_out,
-                                                      unsigned long long* __restrict__ starts,
-                                                      long long* __restrict__ tail, const long long* __restrict__ gv,
-                                                      long long G) {
+__global__ void __launch_bounds__(kCsrBlock) csr_emit(const unsigned long long* k, long long N, long long chunk, int B,
+                                                      long long n, const unsigned long long* base, int* adj,
+                                                      long long* off, long long* m_out, const unsigned long long* starts,
+                                                      long long* tail, const long long* __restrict__ gv, long long G) {
   wait_predecessor();
   const int lane = threadIdx.x & 31;
   GraphBase gb(gv, G);
@@ -524,7 +520,7 @@ __global__ void __launch_bounds__(kCsrBlock) csr_emit(const unsigned long long* 
   if (lo >= hi) return;
   unsigned long long running = base[w];
   WarpKeys t;
-  t.prev = lo > 0 ? __ldg(k + lo - 1) : kSentinel;
+  t.prev = lo > 0 ? k[lo - 1] : kSentinel;
   for (long long ts = lo; ts < hi; ts += kUTile) {
     t.load(k, ts, hi, N, lane);
     // the lookups of each key (kEmitUpper: the lower neighbours of u come
@@ -570,8 +566,8 @@ __global__ void __launch_bounds__(kCsrBlock) csr_emit(const unsigned long long* 
 // endpoint, then sentinels. starts[x] = keys of B whose larger endpoint is
 // below x, for x in [0, n] (cleared beforehand: the groups up to the first key's
 // need no store; the last key records its group in tail[0] and E' in tail[1]).
-__global__ void csr_lower_starts(const unsigned long long* __restrict__ Bq, long long E, int B, long long n,
-                                 unsigned long long* __restrict__ starts, long long* __restrict__ tail) {
+__global__ void csr_lower_starts(const unsigned long long* Bq, long long E, int B, long long n,
+                                 unsigned long long* starts, long long* tail) {
   wait_predecessor();
   constexpr int kU = 4;  // keys per thread per step, all loaded first
   const unsigned long long mask = (1ull << B) - 1;
@@ -582,8 +578,8 @@ __global__ void csr_lower_starts(const unsigned long long* __restrict__ Bq, long
     for (int u = 0; u < kU; u++) {
       const long long i = i0 + u * stride;
       x[u] = i < E ? __ldcs(Bq + i) : kSentinel;
-      xp[u] = i < E && i > 0 ? __ldg(Bq + i - 1) : kSentinel;
-      xn[u] = i + 1 < E ? __ldg(Bq + i + 1) : kSentinel;
+      xp[u] = i < E && i > 0 ? Bq[i - 1] : kSentinel;
+      xn[u] = i + 1 < E ? Bq[i + 1] : kSentinel;
     }
 #pragma unroll
     for (int u = 0; u < kU; u++) {
@@ -603,8 +599,7 @@ __global__ void csr_lower_starts(const unsigned long long* __restrict__ Bq, long
 }
 
 // starts[v] = E' for the groups above the last key's group s = tail[0], in parallel.
-__global__ void csr_fill_starts(const long long* __restrict__ tail, long long n,
-                                unsigned long long* __restrict__ starts) {
+__global__ void csr_fill_starts(const long long* tail, long long n, unsigned long long* starts) {
   wait_predecessor();
   const long long s = tail[0], m_val = tail[1];
   for (long long v = s + 1 + blockIdx.x * (long long)blockDim.x + threadIdx.x; v <= n;
@@ -614,9 +609,9 @@ __global__ void csr_fill_starts(const long long* __restrict__ tail, long long n,
 
 // The lower neighbours: B's key i (u, v) is v's (i - starts[v])-th lower
 // neighbour, and v's list opens with them.
-__global__ void csr_lower_emit(const unsigned long long* __restrict__ Bq, long long E, int B,
-                               const long long* __restrict__ off, const unsigned long long* __restrict__ starts,
-                               int* __restrict__ adj, const long long* __restrict__ gv, long long G) {
+__global__ void csr_lower_emit(const unsigned long long* Bq, long long E, int B, const long long* off,
+                               const unsigned long long* starts, int* adj, const long long* __restrict__ gv,
+                               long long G) {
   wait_predecessor();
   GraphBase gb(gv, G);
   constexpr int kU = 4;  // keys per thread per step, all loaded first, then all their lookups
@@ -632,7 +627,7 @@ __global__ void csr_lower_emit(const unsigned long long* __restrict__ Bq, long l
 #pragma unroll
     for (int u = 0; u < kU; u++) {
       const long long v = (long long)(x[u] & mask);
-      at[u] = x[u] != kSentinel ? (unsigned long long)__ldg(off + v) - __ldg(starts + v) : 0;
+      at[u] = x[u] != kSentinel ? (unsigned long long)off[v] - starts[v] : 0;
     }
 #pragma unroll
     for (int u = 0; u < kU; u++)
@@ -647,8 +642,8 @@ __global__ void csr_lower_emit(const unsigned long long* __restrict__ Bq, long l
 // offsets[v] = (A's unique keys with smaller endpoint below v) + starts[v]:
 // csr_emit<kEmitUpper> wrote the first term for v up to the last valid key's
 // group tail[0]; above it the term is tail[1], A's unique keys in all.
-__global__ void csr_finish_offsets(const long long* __restrict__ tail, long long n, long long* __restrict__ off,
-                                   const unsigned long long* __restrict__ starts) {
+__global__ void csr_finish_offsets(const long long* tail, long long n, long long* off,
+                                   const unsigned long long* starts) {
   wait_predecessor();
   const long long s = tail[0], m_val = tail[1];
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v <= n; v += (long long)gridDim.x * blockDim.x)
@@ -729,7 +724,9 @@ CsrLayout csr_layout(long long n, long long E, int sms, long long max_graph_n, b
 }
 
 // Launches a kernel of the chain. early: it starts while the one before it
-// drains (every kernel of this file begins with wait_predecessor). A list of at
+// drains (every kernel of this file begins with wait_predecessor, and reads what
+// its predecessors wrote by ordinary loads: the read-only path, __ldg or const
+// __restrict__, is for data that stays as it is while the kernel is resident). A list of at
 // most one tile per CTA is some thirty launches of a few microseconds, whose
 // start-up that takes off the critical path: 1.0 M edges 0.310 -> 0.279 ms. A
 // longer list's kernels fill the GPU, and waiting CTAs only take their room
