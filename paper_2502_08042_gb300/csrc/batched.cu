@@ -238,6 +238,10 @@ __device__ __forceinline__ int load_chunk(const GraphDesc& gd, const int* F, int
       const long long e = gd.off[v + 1];
       if (st < 0 || e < st || e > gd.m || e - st >= n) flag_bad(status, 2, v, &sh.bad);
       else len = (int)(e - st);
+      // A vertex peeled at a level above 0 has arcs, except in a graph that is
+      // not symmetric, where a 16-bit d~ can be decremented below 0 and come
+      // round. The map from arcs to lists (chunk_arcs) relies on it.
+      if (len == 0 && k > 0) flag_bad(status, 4, v, &sh.bad);
     } else {
       flag_bad(status, 3, v, &sh.bad);
     }
@@ -263,7 +267,9 @@ __device__ __forceinline__ int load_chunk(const GraphDesc& gd, const int* F, int
 // result is checked (a check that can branch to flag_bad between two loads
 // makes each wait for the one before), and the crossing vertices of kBatchIlp
 // windows are appended to Fn with one atomic. Every list of a chunk holds an
-// arc: a frontier vertex of level k >= 1 has degree >= k.
+// arc (load_chunk reports one that does not): two lists that start at the same
+// arc would count as one in the bit mask, and the arcs after them would be
+// read past their lists' ends.
 template <int BLOCK, int kIlp, int kMode, bool kNarrow>
 __device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& D, int n, int k, int jlo, int jhi,
                                            int cnum, int* Fn, int* counter, int* status, BatchShared<BLOCK>& sh) {

@@ -82,3 +82,29 @@ def test_last_offset_below_the_first_served(cluster):
     for i in (0, 2, 3):
         assert res[t[i]][0] == 49  # (a launch's requests share its status)
         np.testing.assert_array_equal(outs[i], want)
+
+
+@pytest.mark.parametrize("opts", FORMS, ids=str)
+@pytest.mark.parametrize("per", [1, 4])
+def test_arcs_into_a_vertex_without_arcs(opts, per):
+    """Not symmetric: more than 2^16 arcs into the last vertex, which has none
+    of its own. Its 16-bit d~ comes round and lands on the level that many
+    others land on at once; its empty list is reported, and no arc is read for
+    it (its list starts where the arcs end)."""
+    a = 70_000 // per  # vertices of `per` arcs to the last vertex and one to a vertex of a K4, which it lands on level per + 1
+    x = 4 * ((a + 3) // 4)
+    n = a + x + 1
+    block = np.arange(x) // 4 * 4
+    others = np.stack([(np.arange(x) + 1 + j) % 4 for j in range(3)], 1) + block[:, None]
+    pad = np.zeros((x, per - 1), np.int64)  # degree per + 2 = level + 1: arcs to the first vertex, repeated
+    lists = np.concatenate([np.concatenate([np.full((a, per), n - 1), a + np.arange(a)[:, None]], 1).ravel(),
+                            np.concatenate([pad, a + others], 1).ravel()])
+    deg = np.concatenate([np.full(a, per + 1), np.full(x, per + 2), [0]])
+    off = np.concatenate([[0], np.cumsum(deg)])
+    assert off[-1] == len(lists) and off[-2] == off[-1]
+    gv = np.array([0, n], np.int64)
+    with KCore(0, **opts) as k:
+        _, _, err = run_batch(k, gv, off, lists)
+        assert err == "NOT_SIMPLE"
+        nn, s, d = gg.complete(60)
+        assert_parity(k, nn, *oracle.build_csr(nn, s, d))
