@@ -43,6 +43,7 @@
 
 #include "kcore_batched.h"
 #include "kcore_device.cuh"
+#include "kcore_search.h"
 
 namespace kc {
 
@@ -271,20 +272,21 @@ __device__ __forceinline__ int load_chunk(const GraphDesc& gd, const int* F, int
 // arc would count as one in the bit mask, and the arcs after them would be
 // read past their lists' ends.
 template <int BLOCK, int kIlp, int kMode, bool kNarrow>
-__device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& D, int n, int k, int jlo, int jhi,
-                                           int cnum, int* Fn, int* counter, int* status, BatchShared<BLOCK>& sh) {
+__device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& D, int n, int k, unsigned jlo,
+                                           unsigned jhi, int cnum, int* Fn, int* counter, int* status, BatchShared<BLOCK>& sh) {
   constexpr int kW = BLOCK / 32;
   const int lane = threadIdx.x & 31, warp = team_tid<BLOCK>() >> 5;
-  const int run = ((((jhi - jlo + 31) >> 5) + kW - 1) / kW) << 5;  // arcs per warp
-  int j0 = jlo + warp * run;
-  const int jend = min(jhi, j0 + run);
+  // (positions go up to 2^31 - 2, and an iteration's reach past it: unsigned)
+  const unsigned run = ((((jhi - jlo + 31) >> 5) + kW - 1) / kW) << 5;  // arcs per warp
+  unsigned j0 = jlo + warp * run;
+  const unsigned jend = min(jhi, j0 + run);
   if (j0 >= jend || __any_sync(kFull, sh.bad)) return;
   int idx;  // last vertex that starts at or before j0
   {
     const int x = lane * kW;
-    unsigned m = __ballot_sync(kFull, x < cnum && sh.pre[x] <= j0);
+    unsigned m = __ballot_sync(kFull, x < cnum && (unsigned)sh.pre[x] <= j0);
     const int c = m ? (31 - __clz(m)) * kW : 0;
-    m = __ballot_sync(kFull, lane < kW && c + lane < cnum && sh.pre[c + lane] <= j0);
+    m = __ballot_sync(kFull, lane < kW && c + lane < cnum && (unsigned)sh.pre[c + lane] <= j0);
     idx = m ? c + 31 - __clz(m) : c;
   }
   const unsigned le = lanemask_lt() | (1u << lane);
@@ -293,7 +295,7 @@ __device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& 
     // the starts inside the iteration: one read gives the next 32; when they
     // reach past it, the windows' masks do not depend on each other
     const int e0 = idx + 1 + lane;
-    const unsigned d0 = e0 < cnum ? (unsigned)(sh.pre[e0] - j0) : 0x7fffffffu;
+    const unsigned d0 = e0 < cnum ? (unsigned)sh.pre[e0] - j0 : 0x7fffffffu;
     const bool few = __shfl_sync(kFull, d0, 31) >= kIlp * 32u;
 #pragma unroll
     for (int q = 0; q < kIlp; q++) {
@@ -302,16 +304,16 @@ __device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& 
         unsigned d = d0 - q * 32u;
         if (!few) {
           const int e = idx + 1 + lane;
-          d = e < cnum ? (unsigned)(sh.pre[e] - (j0 + q * 32)) : 32u;
+          d = e < cnum ? (unsigned)sh.pre[e] - (j0 + q * 32) : 32u;
         }
         const unsigned m = __reduce_or_sync(kFull, d < 32u ? 1u << d : 0u);
         const int mine = idx + __popc(m & le);
         idx += __popc(m);
-        const int j = j0 + q * 32 + lane;
+        const unsigned j = j0 + q * 32 + lane;
         if (j < jend) u[q] = ld_stream_s32(sh.list[mine] + j);
       }
     }
-    const int left = jend - j0 - lane;
+    const int left = (int)(jend - j0) - lane;
     bool bad = false;  // an id outside [0, n)
 #pragma unroll
     for (int q = 0; q < kIlp; q++) bad |= (unsigned)u[q] >= (unsigned)n;
@@ -348,8 +350,8 @@ __device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& 
 }
 
 template <int BLOCK>
-__device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& D, int n, int k, int jlo, int jhi,
-                                           int cnum, int* Fn, int* counter, int* status, BatchShared<BLOCK>& sh) {
+__device__ __forceinline__ void chunk_arcs(const GraphDesc& gd, const DegStore& D, int n, int k, unsigned jlo,
+                                           unsigned jhi, int cnum, int* Fn, int* counter, int* status, BatchShared<BLOCK>& sh) {
   // at most one window per warp: without the slots of further windows, whose
   // instructions alone would be most of a small graph's phase
 #define KC_ARCS2(ILP, MODE)                                                                                     \
@@ -528,6 +530,7 @@ __device__ void peel_one_graph(int smem_deg_max, int* status, int* sdeg, BatchSh
     return;
   }
   const bool narrow = dmax < 65536;
+  const int chunk = chunk_vertices(BLOCK, dmax);
   const int fit = narrow ? 2 * smem_deg_max : smem_deg_max;  // vertices that fit in shared memory
   const DegStore D{gd.deg, (unsigned)__cvta_generic_to_shared(sdeg), fit,
                    n <= fit ? kDegSmem : (fit > 0 ? kDegSplit : kDegGlobal), narrow, l2_evict_last_policy()};
@@ -550,8 +553,8 @@ __device__ void peel_one_graph(int smem_deg_max, int* status, int* sdeg, BatchSh
     bool fodd = false;  // the frontier is in F1
     while (nf > 0) {
       peeled += nf;
-      for (int c0 = 0; c0 < nf; c0 += BLOCK) {
-        const int cnum = min(BLOCK, nf - c0);
+      for (int c0 = 0; c0 < nf; c0 += chunk) {
+        const int cnum = min(chunk, nf - c0);
         const int total = load_chunk<BLOCK>(gd, (fodd ? gd.F1 : gd.F0) + c0, cnum, n, k, true, status, sh, ph);
         // every thread has read the last subround's counter: clear it for the next
         if (tid == 0 && c0 == 0) sh.cnt[(r + 1) & 1] = 0;
@@ -743,6 +746,7 @@ struct ClusterPeel {
       return;
     }
     const bool narrow = dmax < 65536;
+    const int chunk = chunk_vertices(BLOCK, dmax);
     const DegStore D{gd.deg, 0u, 0, kDegGlobal, narrow, l2_evict_last_policy()};
     // phase: initial induced degrees, the identity active list
     const int nw = narrow ? (n + 1) / 2 : n;
@@ -764,12 +768,11 @@ struct ClusterPeel {
       int* Fc = gd.F0;
       int* Fn = gd.F1;
       while (nf > 0) {
-        // a large frontier: the CTAs take whole chunks of BLOCK frontier
-        // vertices in turn; a small one: every CTA walks every chunk and takes
+        // a large frontier: the CTAs take whole chunks of frontier vertices in turn; a small one: every CTA walks every chunk and takes
         // its share of the chunk's arcs (the first CTA writes their coreness)
-        const bool whole = nf >= 2 * C * BLOCK;
-        for (int c0 = whole ? r * BLOCK : 0; c0 < nf; c0 += whole ? C * BLOCK : BLOCK) {
-          const int cnum = min(BLOCK, nf - c0);
+        const bool whole = nf >= 2 * C * chunk;
+        for (int c0 = whole ? r * chunk : 0; c0 < nf; c0 += whole ? C * chunk : chunk) {
+          const int cnum = min(chunk, nf - c0);
           const int total = load_chunk<BLOCK>(gd, Fc + c0, cnum, n, k, whole || r == 0, status, sh, sp);
           chunk_arcs<BLOCK>(gd, D, n, k, whole ? 0 : (int)part_lo(total), whole ? total : (int)part_hi(total), cnum, Fn,
                             &slot(ph)[0], status, sh);

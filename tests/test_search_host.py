@@ -1,5 +1,7 @@
-"""The binary search step of the CSR check, compiled for the host: lists of
-more than 2^30 entries, whose middle a 32-bit sum of both ends leaves."""
+"""Index arithmetic of the kernels, compiled for the host. The binary search
+step of the CSR check: lists of more than 2^30 entries, whose middle a 32-bit
+sum of both ends leaves. The batched peel's chunks: 1,024 lists of more than
+2^21 arcs, whose 32-bit sum overflows."""
 import os
 import shutil
 import subprocess
@@ -25,7 +27,19 @@ static int search(int len, int x) {
   }
   return 3;
 }
+static int chunks() {
+  for (int block : {256, 512, 1024})
+    for (long long dmax : {0ll, 1ll, 65535ll, 2097151ll, 2097152ll, 4194305ll, 1ll << 30, 2147483645ll}) {
+      const long long c = kc::chunk_vertices(block, (int)dmax);
+      if (c < 1 || c > block || c * dmax > 0x7fffffff || (c < block && (c + 1) * dmax <= 0x7fffffff)) {
+        printf("block %d dmax %lld: %lld\n", block, dmax, c);
+        return 1;
+      }
+    }
+  return 0;
+}
 int main() {
+  if (chunks()) return 1;
   const int lens[] = {1, 2, 3, 32, (1 << 30) - 1, 1 << 30, (1 << 30) + 1, 1500000000, 2147483645};
   for (int len : lens)
     for (int back : {-1, 0, 1, 2, 1000})
@@ -42,7 +56,7 @@ int main() {
 """
 
 
-def test_middle_of_long_lists(tmp_path):
+def test_middle_and_chunks(tmp_path):
     cxx = shutil.which("g++")
     if not cxx:
         pytest.skip("no g++")
@@ -53,7 +67,10 @@ def test_middle_of_long_lists(tmp_path):
     assert r.returncode == 0, r.stdout
 
 
-def test_the_check_uses_it():
+def test_the_kernels_use_them():
     with open(os.path.join(_native.CSRC, "validate.cu")) as f:
         text = f.read()
     assert "middle(lo[q], hi[q])" in text and "(lo[q] + hi[q])" not in text
+    with open(os.path.join(_native.CSRC, "batched.cu")) as f:
+        text = f.read()
+    assert text.count("= chunk_vertices(BLOCK, dmax);") == 2 and text.count("min(chunk, nf - c0)") == 2
