@@ -403,17 +403,16 @@ kcore_status peel_call(kcore_ctx* h, int64_t n, int64_t m, const int64_t* offset
   const int mode = threshold ? 2 : effective_mode(h);
   const int slice =
       h->opt[KCORE_OPT_SLICE_ARCS] > 0 ? (int)h->opt[KCORE_OPT_SLICE_ARCS] : (mode == 1 ? 512 : kc::kSliceDefault);
-  // (a k'-core query of a small graph or a small k' has no pass heavy enough for
-  // the batch update: clearing its counts would add 5 us to some 65)
-  bool hybrid = mode == 2 && h->opt[KCORE_OPT_BATCH_UPDATE] != 0 &&
-                (threshold ? m >= ((int64_t)1 << 22) && kprime >= 16 : h->opt[KCORE_OPT_LEVEL_WINDOW] == 0);
+  // A k'-core query counts in its output array, so it needs no room for counts
+  // and clears none. In a small graph's heavy passes the second barrier costs
+  // more than the returning atomics (R-MAT, k' = 128, us, without / with the
+  // batch update: 1.0 M edges 82 / 92, 2.1 M 71.5 / 72.7, 16.8 M 279 / 168), and
+  // a small k' has no heavy pass.
+  const bool hybrid = mode == 2 && h->opt[KCORE_OPT_BATCH_UPDATE] != 0 &&
+                      (threshold ? m >= ((int64_t)1 << 22) && kprime >= 16 : h->opt[KCORE_OPT_LEVEL_WINDOW] == 0);
+  const bool counts = mode == 3 || (hybrid && !threshold);
   const bool sample = sampling_on(h, threshold);
-  PeelLayout L = peel_layout(n, m, slice, mode == 3 || hybrid, sample);
-  if (threshold && h->ws_external && h->ws_bytes < L.total) {
-    // a caller's workspace without room for the counts: the query needs none
-    hybrid = false;
-    L = peel_layout(n, m, slice, false, sample);
-  }
+  const PeelLayout L = peel_layout(n, m, slice, counts, sample);
   kcore_status st = ensure_ws(h, L.total);
   if (st != KCORE_OK) return st;
   char* ws = (char*)h->ws;
@@ -449,7 +448,7 @@ kcore_status peel_call(kcore_ctx* h, int64_t n, int64_t m, const int64_t* offset
   a.window = mode == 2 && !threshold ? (int)h->opt[KCORE_OPT_LEVEL_WINDOW] : 0;
   a.hybrid = hybrid ? 1 : 0;
   a.A2 = (int*)(ws + L.a2);
-  a.hcnt = (int*)(ws + L.hcnt);
+  a.hcnt = threshold ? out : (int*)(ws + L.hcnt);
   a.touched = (int*)(ws + L.touched);
   a.kprime = threshold ? std::max<int32_t>(kprime, 0) : 0;
   a.size_out = (long long*)size_out;
@@ -480,7 +479,7 @@ kcore_status peel_call(kcore_ctx* h, int64_t n, int64_t m, const int64_t* offset
   if (a.trace && (e = cudaMemsetAsync(a.trace, 0, 8 * (size_t)kc::kTraceFields * (size_t)L.max_rounds,
                                       stream)) != cudaSuccess)
     return cuda_fail(h, e, "memset trace");
-  if ((mode == 3 || hybrid) && (e = cudaMemsetAsync(a.hcnt, 0, 4 * (size_t)n, stream)) != cudaSuccess)
+  if (counts && (e = cudaMemsetAsync(a.hcnt, 0, 4 * (size_t)n, stream)) != cudaSuccess)
     return cuda_fail(h, e, "memset counts");
   h->last_ctl2 = nullptr;
   if (sample) {

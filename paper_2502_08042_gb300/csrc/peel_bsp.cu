@@ -1079,12 +1079,13 @@ __device__ void run_hist(const PeelArgs& a, Shared& sh, const PassCtx& pc, unsig
 }
 
 // Apply phase over list[0, nt) (the touched list, or the active list, where
-// untouched vertices have count 0): a warp handles 32 vertices at a time.
+// untouched vertices have count 0): a warp handles 32 vertices at a time. A
+// k'-core query counts in core[] itself, whose vertices above the level hold 1.
 __device__ void run_apply(const PeelArgs& a, const PassCtx& pc, const int* list, unsigned long long nt) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned long long gw = (unsigned long long)blockIdx.x * kWarps + warp;
   const unsigned long long nw = (unsigned long long)gridDim.x * kWarps;
-  const int t = pc.t;
+  const int t = pc.t, none = a.threshold ? 1 : 0;
   for (unsigned long long base = gw * kWarp; base < nt; base += nw * kWarp) {
     const unsigned long long i = base + lane;
     int u = -1;
@@ -1094,9 +1095,10 @@ __device__ void run_apply(const PeelArgs& a, const PassCtx& pc, const int* list,
     if (i < nt) {
       u = __ldcg(list + i);
       if ((unsigned)u < (unsigned)a.n) {
-        const int f = __ldcg(a.hcnt + u);
-        if (f) a.hcnt[u] = 0;
+        const int cnt = __ldcg(a.hcnt + u);
         const int old = __ldcg(a.deg + u);
+        const int f = old > t ? cnt - none : 0;  // only vertices above the level were counted
+        if (f) a.hcnt[u] = none;
         a.deg[u] = old - f;
         cross = old > t && old - f <= t;
         if (cross) {
