@@ -22,7 +22,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <cmath>
 #include <cstring>
 #include <map>
 #include <string>
@@ -85,7 +84,7 @@ struct Request {
   int64_t ticket = 0;
   int64_t n = 0, m = 0;
   int32_t* core_h = nullptr;
-  bool large = false, compact = false;
+  bool large = false;
   size_t pool_off = 0, pool_bytes = 0;
   char* d = nullptr;  // device base of the request's pool block
   size_t o_off = 0, o_adj = 0, o_core = 0, o_kmax = 0, o_state = 0;
@@ -146,31 +145,26 @@ struct DevGuard {
   }
 };
 
-long long isqrt_s(long long m) {
-  long long r = (long long)std::sqrt((double)m);
-  while (r > 0 && r * r > m) r--;
-  while ((r + 1) * (r + 1) <= m) r++;
-  return r;
-}
-
-// Whole-GPU peel workspace for a large request (same layout as the handle's):
-// for the default schedule, or (compact) without the batch update's counts and
-// with longer slices, for a request that the pool admits only so.
+// Whole-GPU peel workspace for a large request. What a request holds of the
+// pool decides how many are admitted beside it: at most a queue of 64-arc
+// slices and 2 sqrt(m) round records of 512 bytes. The peel needs a ring of
+// three records, and the rest pays for 32-arc slices (m / 8 bytes) up to 2^26
+// arcs. R-MAT of 2^20 + 1 vertices, ms per peel: 32 arcs 8.53, 64 arcs 8.97 (the batch update's
+// counts would change nothing there: 8.58).
 struct LargeLayout {
-  size_t ctl, rounds, deg, a0, a1, q, hcnt, total;
+  size_t ctl, rounds, deg, a0, a1, q, total;
   long long qcap;
-  int max_rounds, slice;
+  int slice;
 };
-LargeLayout large_layout(long long n, long long m, bool compact) {
+LargeLayout large_layout(long long n, long long m) {
   LargeLayout L{};
-  L.slice = compact ? 64 : kc::kSliceDefault;
+  L.slice = m <= 1ll << 26 ? kc::kSliceDefault : 2 * kc::kSliceDefault;
   L.qcap = n + (m + L.slice - 1) / L.slice + 1;
-  L.max_rounds = (int)std::min<long long>(2 * isqrt_s(m) + 8, 2 * n + 8);
   size_t o = 0;
   L.ctl = o;
   o = al256(o + sizeof(kc::PeelCtl));
   L.rounds = o;
-  o = al256(o + sizeof(kc::RoundRec) * (size_t)L.max_rounds);
+  o = al256(o + sizeof(kc::RoundRec) * (size_t)kc::kPhaseRing);
   L.deg = o;
   o = al256(o + 4 * (size_t)n);
   L.a0 = o;
@@ -179,8 +173,6 @@ LargeLayout large_layout(long long n, long long m, bool compact) {
   o = al256(o + 4 * (size_t)n);
   L.q = o;
   o = al256(o + 8 * (size_t)L.qcap);
-  L.hcnt = o;
-  if (!compact) o = al256(o + 4 * (size_t)n);
   L.total = o;
   return L;
 }
@@ -307,14 +299,10 @@ kcore_status kcore_server_submit(kcore_server s, int64_t n, int64_t m, const int
   r.o_kmax = o;
   o = al256(o + 8);
   r.o_state = o;
-  if (r.large) o += large_layout(n, m, false).total;
+  if (r.large) o += large_layout(n, m).total;
   else o += 5 * al256(4 * (size_t)std::max<int64_t>(n, 1));
   size_t poff = 0;
-  if (!s->alloc->alloc(o, &poff)) {
-    r.compact = r.large;
-    if (r.compact) o = r.o_state + large_layout(n, m, true).total;
-    if (!r.compact || !s->alloc->alloc(o, &poff)) return KCORE_ERR_CAPACITY;  // not admitted now
-  }
+  if (!s->alloc->alloc(o, &poff)) return KCORE_ERR_CAPACITY;  // not admitted now
   r.pool_off = poff;
   r.pool_bytes = o;
   r.d = s->pool + poff;
@@ -436,7 +424,7 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
   for (auto& kv : s->reqs) {
     Request& r = kv.second;
     if (r.state != RS_READY || !r.large) continue;
-    LargeLayout L = large_layout(r.n, r.m, r.compact);
+    LargeLayout L = large_layout(r.n, r.m);
     char* ws = r.d + r.o_state;
     kc::PeelArgs a{};
     a.n = r.n;
@@ -451,7 +439,7 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
     a.Q = (unsigned long long*)(ws + L.q);
     a.qcap = L.qcap;
     a.rounds = (kc::RoundRec*)(ws + L.rounds);
-    a.max_rounds = L.max_rounds;
+    a.max_rounds = kc::kPhaseRing;  // bounds trace records only; no trace is written here
     a.ctl = (kc::PeelCtl*)(ws + L.ctl);
     // the handle's default schedule
     a.slice = L.slice;
@@ -467,10 +455,7 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
     a.take_div = grid * (kc::bsp_block_size() / 32);
     a.local_batches = kc::kLocalBatchesDefault;
     a.precheck_items = kc::kPrecheckDefault;
-    a.hybrid = r.compact ? 0 : 1;
-    a.hcnt = (int*)(ws + L.hcnt);
     e = cudaMemsetAsync(ws, 0, L.deg, s->large);
-    if (e == cudaSuccess && a.hybrid) e = cudaMemsetAsync(a.hcnt, 0, 4 * (size_t)r.n, s->large);
     if (e == cudaSuccess) e = kc::bsp_launch(a, grid, s->large);
     if (e == cudaSuccess) e = cudaEventRecord(r.ev, s->large);
     if (e != cudaSuccess) {
@@ -499,7 +484,7 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
   for (auto& kv : s->reqs) {
     Request& r = kv.second;
     if (r.state != RS_RUNNING || !r.large || cudaEventQuery(r.ev) != cudaSuccess) continue;
-    LargeLayout L = large_layout(r.n, r.m, r.compact);
+    LargeLayout L = large_layout(r.n, r.m);
     char* ws = r.d + r.o_state;
     if (r.n > 0) cudaMemcpyAsync(r.core_h, r.d + r.o_core, 4 * (size_t)r.n, cudaMemcpyDeviceToHost, s->copy);
     cudaMemcpyAsync(r.kmax_slot, r.d + r.o_kmax, 4, cudaMemcpyDeviceToHost, s->copy);
