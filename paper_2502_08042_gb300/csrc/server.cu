@@ -102,7 +102,8 @@ struct Batch {
   cudaEvent_t done = nullptr;
   int* d_status = nullptr;
   int stream = 0;  // launch stream
-  bool finished = false;
+  bool ended = false;     // the launch has run: its stream is free
+  bool finished = false;  // its results are being copied back
 };
 
 }  // namespace
@@ -149,8 +150,8 @@ struct DevGuard {
 // pool decides how many are admitted beside it: at most a queue of 64-arc
 // slices and 2 sqrt(m) round records of 512 bytes. The peel needs a ring of
 // three records, and the rest pays for 32-arc slices (m / 8 bytes) up to 2^26
-// arcs. R-MAT of 2^20 + 1 vertices, ms per peel: 32 arcs 8.53, 64 arcs 8.97 (the batch update's
-// counts would change nothing there: 8.58).
+// arcs. R-MAT of 2^20 + 1 vertices, ms per peel: 32 arcs 8.53, 64 arcs 8.97
+// (the batch update's counts would change nothing there: 8.58).
 struct LargeLayout {
   size_t ctl, rounds, deg, a0, a1, q, total;
   long long qcap;
@@ -366,6 +367,16 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
     if (r.state == RS_COPYING && cudaEventQuery(r.ev) == cudaSuccess) r.state = RS_READY;
     if (r.state == RS_READY && !r.large) small_ready.push_back(r.ticket);
   }
+  // launches that have run free their streams for the requests ready now (a
+  // caller that polls seldom would wait a poll longer otherwise)
+  auto ended = [s](Batch& b) {
+    if (!b.ended && cudaEventQuery(b.done) == cudaSuccess) {
+      b.ended = true;
+      s->stream_busy[b.stream] = false;
+    }
+    return b.ended;
+  };
+  for (auto& kv : s->batches) ended(kv.second);
   cudaGetLastError();  // cudaEventQuery's cudaErrorNotReady is not an error
   // 2a. batched launches for the small requests that became ready together,
   // one in flight per launch stream: behind a running launch the requests
@@ -469,9 +480,8 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
   // 3. finished launches -> copy results back
   for (auto& kv : s->batches) {
     Batch& b = kv.second;
-    if (b.finished || cudaEventQuery(b.done) != cudaSuccess) continue;
+    if (b.finished || !ended(b)) continue;
     b.finished = true;
-    s->stream_busy[b.stream] = false;
     for (int64_t t : b.reqs) {
       Request& r = s->reqs[t];
       if (r.n > 0) cudaMemcpyAsync(r.core_h, r.d + r.o_core, 4 * (size_t)r.n, cudaMemcpyDeviceToHost, s->copy);

@@ -33,3 +33,28 @@ def test_two_large_requests_fit():
     for x, c in zip(t, outs):
         assert res[x] == (int(want.max()), 0)
         np.testing.assert_array_equal(c, want)
+
+
+def test_a_poll_launches_on_the_stream_it_finds_finished():
+    """One launch stream: the poll that finds its launch finished also launches
+    the request that became ready meanwhile."""
+    n, s, d = gg.complete(50)
+    off, adj = oracle.build_csr(n, s, d)
+    outs = [np.full(n, -9, np.int32) for _ in range(2)]
+
+    def poll(srv):
+        got = [t for t, _, _ in srv.poll()]
+        torch.cuda.synchronize()
+        return got
+
+    with KCoreServer(0, pool_bytes=1 << 26, streams=1) as srv:
+        a = srv.submit(off, adj, outs[0])
+        torch.cuda.synchronize()
+        assert poll(srv) == []  # launches a
+        b = srv.submit(off, adj, outs[1])
+        torch.cuda.synchronize()
+        assert poll(srv) == []   # a's results; launches b
+        assert poll(srv) == [a]  # b's results
+        assert poll(srv) == [b]
+    for c in outs:
+        np.testing.assert_array_equal(c, 49)
