@@ -840,10 +840,14 @@ kcore_status kcore_build_csr_batched(kcore_handle h, int64_t num_graphs, int64_t
   h->pending = true;
   h->last_validate_status = nullptr;
   kc::CsrLayout L = kc::csr_layout(total_vertices, num_edges, h->sms, max_graph_vertices);
-  // a caller's workspace without room for the edge route's list starts takes the arc route
-  if (h->ws_external && h->ws_bytes < L.total)
-    L = kc::csr_layout(total_vertices, num_edges, h->sms, max_graph_vertices, false);
+  // without room for the edge route's list starts, in a caller's workspace or in
+  // what the device has left, the arc route
   kcore_status st = ensure_ws(h, L.total);
+  if (st == KCORE_ERR_OOM && L.by_edges) {
+    h->err.clear();
+    L = kc::csr_layout(total_vertices, num_edges, h->sms, max_graph_vertices, false);
+    st = ensure_ws(h, L.total);
+  }
   if (st != KCORE_OK) return st;
   cudaError_t e = kc::csr_build_launch(L, (char*)h->ws, total_vertices, num_edges, src, dst,
                                        (const long long*)graph_vertex_offsets,
