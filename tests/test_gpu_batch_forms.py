@@ -70,3 +70,14 @@ def test_wide_degrees(sv):
     batch = segmented([(n, np.concatenate([s, e[0]]), np.concatenate([d, e[1]]))])
     with KCore(0, batch_smem_vertices=min(sv, 50000)) as k:
         check(k, batch)
+
+
+@pytest.mark.parametrize("sv", [0, 1, 30_001, 50_000])
+def test_wide_degrees_split(sv):
+    """The same hub with the first sv vertices' 32-bit degrees in shared memory.
+    (No graph with a degree of 2^16 fits there as a whole.)"""
+    n, s, d = gg.star(70001)
+    e = gg.er(n, 100000, seed=6)
+    batch = segmented([(n, np.concatenate([s, e[0]]), np.concatenate([d, e[1]]))])
+    with KCore(0, batch_smem_vertices=sv) as k:
+        check(k, batch)
