@@ -357,10 +357,11 @@ __global__ void __launch_bounds__(kCsrBlock, 3) rs_downsweep(const unsigned long
     __syncthreads();
     // A key's rank among its warp's keys of the same digit, in key order (rows
     // in order, lanes in order within a row). The lanes of a digit find each
-    // other by or-ing their bits into its counter and reading it back: about 11
-    // cycles of the SM per row of 32 random digits, where match.any takes 40
-    // and eight ballots 16 (one CTA of 256 threads x 5 per SM, measured). The
-    // first pass of a build need not be stable: a counter's old value is rank enough.
+    // other by or-ing their bits into its counter and reading it back (a method
+    // of public GPU radix sorts, CUB's among them): about 11 cycles of the SM
+    // per row of 32 random digits, where match.any takes 40 and eight ballots 16
+    // (one CTA of 256 threads x 5 per SM, measured). The first pass of a build
+    // need not be stable: a counter's old value is rank enough.
 #pragma unroll
     for (int it = 0; it < kSortKeys; it++) {
       const bool v = valid(it);
@@ -702,13 +703,11 @@ CsrLayout csr_layout(long long n, long long E, int sms, long long max_graph_n, b
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   L.status = off;
   off = al(off + 256);
-  // two spare keys per buffer: a single graph's build keeps two sequences of
-  // E keys per buffer, the second from an even index, and a 16-byte copy may
-  // read the key after a sequence's last
+  // 2E keys per buffer: the arc route's sequence, or the edge route's two
   L.keys0 = off;
-  off = al(off + 8 * (size_t)(N + 2));
+  off = al(off + 8 * (size_t)N);
   L.keys1 = off;
-  off = al(off + 8 * (size_t)(N + 2));
+  off = al(off + 8 * (size_t)N);
   // sized for 2E keys on either route: a batch's workspace is at most a single graph's
   const size_t counts = std::max<size_t>(256 * (size_t)ctas_of(N), (size_t)warps_of(N) + kCsrBlock / 32);
   L.hist = off;
@@ -795,10 +794,8 @@ cudaError_t csr_build_launch(const CsrLayout& L, char* ws, long long n, long lon
   if (L.by_edges) {
     // the edge route: A = the E edge keys sorted by (min, max); B = A stably
     // sorted by max. A ping-pongs between the first halves of the two key
-    // buffers, B between their second halves (from an even index: 16-byte
-    // copies stay aligned)
-    const long long off2 = (E + 1) / 2 * 2;
-    unsigned long long *a0 = k0, *a1 = k1, *b0 = k0 + off2, *b1 = k1 + off2;
+    // buffers, B between their second halves
+    unsigned long long *a0 = k0, *a1 = k1, *b0 = k0 + E, *b1 = k1 + E;
     const int passes_a = (2 * L.B + 7) / 8;
     for (int p = 0; p < passes_a; p++) {
       pass(p == 0 ? (gv ? kCanonB : kCanon) : kKeys, a0, a1, E, L.chunk, 8 * p, 0xff);
