@@ -42,19 +42,21 @@ def test_a_poll_launches_on_the_stream_it_finds_finished():
     off, adj = oracle.build_csr(n, s, d)
     outs = [np.full(n, -9, np.int32) for _ in range(2)]
 
-    def poll(srv):
-        got = [t for t, _, _ in srv.poll()]
-        torch.cuda.synchronize()
-        return got
-
     with KCoreServer(0, pool_bytes=1 << 26, streams=1) as srv:
+        got = []
+
+        def poll():
+            got.extend(t for t, _, _ in srv.poll())
+            torch.cuda.synchronize()
+
         a = srv.submit(off, adj, outs[0])
         torch.cuda.synchronize()
-        assert poll(srv) == []  # launches a
+        poll()  # launches a
         b = srv.submit(off, adj, outs[1])
         torch.cuda.synchronize()
-        assert poll(srv) == []   # a's results; launches b
-        assert poll(srv) == [a]  # b's results
-        assert poll(srv) == [b]
-    for c in outs:
-        np.testing.assert_array_equal(c, 49)
+        poll()  # finds a finished; launches b
+        poll()  # finds b finished: its results are copied back
+        np.testing.assert_array_equal(outs[1], 49)
+        poll()
+        assert sorted(got) == [a, b]
+    np.testing.assert_array_equal(outs[0], 49)
