@@ -136,8 +136,8 @@ struct PeelArgs {
   int kprime;
   long long* size_out;  // optional: the k'-core's vertex count
   // offline subrounds (sync mode 3, Algorithm 2): per-vertex decrement
-  // counts (zero at launch, left zero; a k'-core query: core, whose kept
-  // vertices hold 1) and the touched list of a subround
+  // counts (zero at launch, left zero; or core, zero at launch, in which a
+  // k'-core query counts up from 1) and the touched list of a subround
   int offline;
   int* hcnt;
   int* touched;

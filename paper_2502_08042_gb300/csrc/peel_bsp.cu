@@ -1079,8 +1079,10 @@ __device__ void run_hist(const PeelArgs& a, Shared& sh, const PassCtx& pc, unsig
 }
 
 // Apply phase over list[0, nt) (the touched list, or the active list, where
-// untouched vertices have count 0): a warp handles 32 vertices at a time. A
-// k'-core query counts in core[] itself, whose vertices above the level hold 1.
+// untouched vertices have count 0): a warp handles 32 vertices at a time.
+// hcnt may be core[] itself: a vertex is counted while it is above the level,
+// and its coreness is written when it leaves (a k'-core query's vertices above
+// the level hold 1 there, and counts go on top).
 __device__ void run_apply(const PeelArgs& a, const PassCtx& pc, const int* list, unsigned long long nt) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned long long gw = (unsigned long long)blockIdx.x * kWarps + warp;

@@ -148,10 +148,13 @@ struct DevGuard {
 
 // Whole-GPU peel workspace for a large request. What a request holds of the
 // pool decides how many are admitted beside it: at most a queue of 64-arc
-// slices and 2 sqrt(m) round records of 512 bytes. The peel needs a ring of
-// three records, and the rest pays for 32-arc slices (m / 8 bytes) up to 2^26
-// arcs. R-MAT of 2^20 + 1 vertices, ms per peel: 32 arcs 8.53, 64 arcs 8.97
-// (the batch update's counts would change nothing there: 8.58).
+// slices and 2 sqrt(m) + 8 round records of 512 bytes. The peel needs a ring of
+// three records, and the others' room holds the queue of 32-arc slices (m / 8
+// bytes more) up to 2^26 arcs. R-MAT of 2^20 + 1 / 2^22 / 2^24 vertices, ms per
+// peel: 32 arcs 8.53 / 6.59 / 12.45, 64 arcs 8.97 / 6.67 / 12.84; lengths between
+// them fill 32-lane windows badly (40 arcs: 6.75 at 2^22). The batch update's
+// counts are kept in the coreness array, which nothing reads before a vertex is
+// peeled (R-MAT 24 without it: 12.67).
 struct LargeLayout {
   size_t ctl, rounds, deg, a0, a1, q, total;
   long long qcap;
@@ -466,7 +469,10 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
     a.take_div = grid * (kc::bsp_block_size() / 32);
     a.local_batches = kc::kLocalBatchesDefault;
     a.precheck_items = kc::kPrecheckDefault;
+    a.hybrid = 1;
+    a.hcnt = a.core;
     e = cudaMemsetAsync(ws, 0, L.deg, s->large);
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.hcnt, 0, 4 * (size_t)r.n, s->large);
     if (e == cudaSuccess) e = kc::bsp_launch(a, grid, s->large);
     if (e == cudaSuccess) e = cudaEventRecord(r.ev, s->large);
     if (e != cudaSuccess) {
