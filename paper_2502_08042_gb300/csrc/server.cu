@@ -102,8 +102,7 @@ struct Batch {
   cudaEvent_t done = nullptr;
   int* d_status = nullptr;
   int stream = 0;  // launch stream
-  bool ended = false;     // the launch has run: its stream is free
-  bool finished = false;  // its results are being copied back
+  bool finished = false;
 };
 
 }  // namespace
@@ -189,6 +188,72 @@ void release_request(kcore_server_ctx* s, Request& r) {
   if (r.slot >= 0) s->free_slots.push_back(r.slot);
   r.slot = -1;
   r.kmax_slot = r.status_slot = nullptr;
+}
+
+// Requests whose copies have finished become ready, and the small ones go out.
+kcore_status launch_small(kcore_server_ctx* s) {
+  cudaError_t e;
+  std::vector<int64_t> small_ready;
+  for (auto& kv : s->reqs) {
+    Request& r = kv.second;
+    if (r.state == RS_COPYING && cudaEventQuery(r.ev) == cudaSuccess) r.state = RS_READY;
+    if (r.state == RS_READY && !r.large) small_ready.push_back(r.ticket);
+  }
+  cudaGetLastError();  // cudaEventQuery's cudaErrorNotReady is not an error
+  // batched launches for the small requests that became ready together,
+  // one in flight per launch stream: behind a running launch the requests
+  // would wait all the same, and those that gather meanwhile make one launch
+  // that fills the GPU instead of a queue of launches of a few graphs each.
+  for (size_t first = 0; first < small_ready.size(); first += kc::kMaxSlotsPerLaunch) {
+    size_t idle = 0;
+    while (idle < s->launch.size() && s->stream_busy[idle]) idle++;
+    if (idle == s->launch.size()) break;
+    int cnt = (int)std::min<size_t>(small_ready.size() - first, (size_t)kc::kMaxSlotsPerLaunch);
+    Batch b;
+    if (!s->alloc->alloc(256, &b.pool_off)) break;  // no room for the counters now: next poll
+    b.pool_bytes = 256;
+    int* ctr = (int*)(s->pool + b.pool_off);
+    b.d_status = ctr + 1;
+    kc::SlotList list;
+    list.count = cnt;
+    // largest first: with clusters the cluster-sized graphs lead the list
+    std::vector<std::pair<long long, int64_t>> by_arcs;
+    long long launch_arcs = 0;
+    for (int i = 0; i < cnt; i++) {
+      const Request& r = s->reqs[small_ready[first + i]];
+      by_arcs.push_back({-(long long)r.m, small_ready[first + i]});
+      launch_arcs += (long long)r.m;
+    }
+    std::sort(by_arcs.begin(), by_arcs.end());
+    for (int i = 0; i < cnt; i++) {
+      Request& r = s->reqs[by_arcs[i].second];
+      list.slot[i] = r.slot;
+      r.state = RS_RUNNING;
+      r.batch = s->next_batch;
+      b.reqs.push_back(r.ticket);
+    }
+    cudaStream_t st = s->launch[idle];
+    const int cl = s->cfg.batch_cluster > 1 ? s->cfg.batch_cluster : 0;
+    int grid = std::min(cl ? cnt * cl : cnt, s->desc_grid_cap);
+    long long big = s->cfg.batch_big_arcs > 0 ? (long long)s->cfg.batch_big_arcs
+                                              : std::max<long long>(1, launch_arcs / std::max(grid, 1));
+    e = cudaMemsetAsync(ctr, 0, 2 * sizeof(int), st);
+    if (e == cudaSuccess)
+      e = kc::desc_launch(s->d_table, list, ctr, (int)s->smem_vertices, b.d_status, grid,
+                          s->smem_vertices * 4, st, std::max<long long>(1, launch_arcs / std::max(grid, 1) / 2), cl,
+                          big);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(b.done, st);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      s->err = std::string("batched launch: ") + cudaGetErrorString(e);
+      return KCORE_ERR_CUDA;
+    }
+    b.stream = (int)idle;
+    s->stream_busy[idle] = true;
+    s->batches.emplace(s->next_batch++, b);
+  }
+  return KCORE_OK;
 }
 
 }  // namespace
@@ -363,77 +428,9 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
   *n_out = 0;
   DevGuard g(s->device);
   cudaError_t e;
-  // 1. copies finished -> ready
-  std::vector<int64_t> small_ready;
-  for (auto& kv : s->reqs) {
-    Request& r = kv.second;
-    if (r.state == RS_COPYING && cudaEventQuery(r.ev) == cudaSuccess) r.state = RS_READY;
-    if (r.state == RS_READY && !r.large) small_ready.push_back(r.ticket);
-  }
-  // launches that have run free their streams for the requests ready now (a
-  // caller that polls seldom would wait a poll longer otherwise)
-  auto ended = [s](Batch& b) {
-    if (!b.ended && cudaEventQuery(b.done) == cudaSuccess) {
-      b.ended = true;
-      s->stream_busy[b.stream] = false;
-    }
-    return b.ended;
-  };
-  for (auto& kv : s->batches) ended(kv.second);
-  cudaGetLastError();  // cudaEventQuery's cudaErrorNotReady is not an error
-  // 2a. batched launches for the small requests that became ready together,
-  // one in flight per launch stream: behind a running launch the requests
-  // would wait all the same, and those that gather meanwhile make one launch
-  // that fills the GPU instead of a queue of launches of a few graphs each.
-  for (size_t first = 0; first < small_ready.size(); first += kc::kMaxSlotsPerLaunch) {
-    size_t idle = 0;
-    while (idle < s->launch.size() && s->stream_busy[idle]) idle++;
-    if (idle == s->launch.size()) break;
-    int cnt = (int)std::min<size_t>(small_ready.size() - first, (size_t)kc::kMaxSlotsPerLaunch);
-    Batch b;
-    if (!s->alloc->alloc(256, &b.pool_off)) break;  // no room for the counters now: next poll
-    b.pool_bytes = 256;
-    int* ctr = (int*)(s->pool + b.pool_off);
-    b.d_status = ctr + 1;
-    kc::SlotList list;
-    list.count = cnt;
-    // largest first: with clusters the cluster-sized graphs lead the list
-    std::vector<std::pair<long long, int64_t>> by_arcs;
-    long long launch_arcs = 0;
-    for (int i = 0; i < cnt; i++) {
-      const Request& r = s->reqs[small_ready[first + i]];
-      by_arcs.push_back({-(long long)r.m, small_ready[first + i]});
-      launch_arcs += (long long)r.m;
-    }
-    std::sort(by_arcs.begin(), by_arcs.end());
-    for (int i = 0; i < cnt; i++) {
-      Request& r = s->reqs[by_arcs[i].second];
-      list.slot[i] = r.slot;
-      r.state = RS_RUNNING;
-      r.batch = s->next_batch;
-      b.reqs.push_back(r.ticket);
-    }
-    cudaStream_t st = s->launch[idle];
-    const int cl = s->cfg.batch_cluster > 1 ? s->cfg.batch_cluster : 0;
-    int grid = std::min(cl ? cnt * cl : cnt, s->desc_grid_cap);
-    long long big = s->cfg.batch_big_arcs > 0 ? (long long)s->cfg.batch_big_arcs
-                                              : std::max<long long>(1, launch_arcs / std::max(grid, 1));
-    e = cudaMemsetAsync(ctr, 0, 2 * sizeof(int), st);
-    if (e == cudaSuccess)
-      e = kc::desc_launch(s->d_table, list, ctr, (int)s->smem_vertices, b.d_status, grid,
-                          s->smem_vertices * 4, st, std::max<long long>(1, launch_arcs / std::max(grid, 1) / 2), cl,
-                          big);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventRecord(b.done, st);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      s->err = std::string("batched launch: ") + cudaGetErrorString(e);
-      return KCORE_ERR_CUDA;
-    }
-    b.stream = (int)idle;
-    s->stream_busy[idle] = true;
-    s->batches.emplace(s->next_batch++, b);
-  }
+  // 1, 2a. copies finished -> ready; batched launches
+  kcore_status st = launch_small(s);
+  if (st != KCORE_OK) return st;
   // 2b. large requests: the whole-GPU single-graph peel, one at a time on its stream
   for (auto& kv : s->reqs) {
     Request& r = kv.second;
@@ -484,10 +481,13 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
     r.batch = -1;
   }
   // 3. finished launches -> copy results back
+  bool freed = false;
   for (auto& kv : s->batches) {
     Batch& b = kv.second;
-    if (b.finished || !ended(b)) continue;
+    if (b.finished || cudaEventQuery(b.done) != cudaSuccess) continue;
     b.finished = true;
+    s->stream_busy[b.stream] = false;
+    freed = true;
     for (int64_t t : b.reqs) {
       Request& r = s->reqs[t];
       if (r.n > 0) cudaMemcpyAsync(r.core_h, r.d + r.o_core, 4 * (size_t)r.n, cudaMemcpyDeviceToHost, s->copy);
@@ -509,6 +509,11 @@ kcore_status kcore_server_poll(kcore_server s, int64_t* tickets_out, int32_t* km
     r.state = RS_RESULTS;
   }
   cudaGetLastError();
+  // the requests that waited for a stream go out now, not at the next poll (a
+  // caller may poll seldom); after the results' copies, so that as many as a
+  // next poll would find go out together (before them: 3% fewer graphs/s at
+  // saturation)
+  if (freed && (st = launch_small(s)) != KCORE_OK) return st;
   // 4. results copied -> done
   std::vector<int64_t> done;
   for (auto& kv : s->reqs) {
