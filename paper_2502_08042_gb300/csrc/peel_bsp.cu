@@ -1613,12 +1613,12 @@ __global__ void __launch_bounds__(kBlock, 2) peel_bsp(PeelArgs a) {
         // vertex by its owner). Reductions need no return trip and run at
         // about 1.5x the rate of returning atomics on this GPU; the apply
         // walk costs one pass over the active list and a second barrier.
-        // Measured on R-MAT 24 / R-MAT 22 / kNN: -2.7% / -0.5% / -1.4%.
+        // Measured on R-MAT 24 / R-MAT 22 / kNN: -3.1% / -0.1% / -3.6%.
         // A k'-core query's frontier holds lists of fewer than kprime arcs,
         // and its list all the vertices kept: there the arcs must outnumber
         // them 64 to one. R-MAT 24, returning atomics / batch update, ms:
-        // k' = 16 (up to 40 arcs per vertex kept) 0.48 / 0.62, 128 (580) 2.07 /
-        // 1.43, 512 (9,000) 3.95 / 2.45.
+        // k' = 16 (up to 40 arcs per vertex kept) 0.48 / 0.62, 128 (580) 2.06 /
+        // 1.40, 512 (9,000) 3.91 / 2.35.
         reset_next();
         RoundRec* P = rec();
         const PassCtx hc{P, qend, t, t, false, -1, nullptr, 0};
