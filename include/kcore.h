@@ -304,7 +304,8 @@ kcore_status kcore_build_csr_workspace_size(kcore_handle h, int64_t n, int64_t n
  * KCORE_OPT_BATCH_CLUSTER, the graphs above KCORE_OPT_BATCH_BIG_ARCS arcs by a
  * thread-block cluster each, induced degrees in L2). Uses
  * kcore_batched_workspace_size bytes of workspace (20 bytes per vertex).
- * Malformed offsets or ids are reported as KCORE_ERR_NOT_SIMPLE by
+ * Malformed offsets or ids, and a vertex without arcs that a graph that is not
+ * symmetric brings to a level above 0, are reported as KCORE_ERR_NOT_SIMPLE by
  * kcore_sync_status. */
 kcore_status kcore_decompose_batched(kcore_handle h, int64_t num_graphs, int64_t total_vertices,
                                      int64_t total_arcs, const int64_t* graph_vertex_offsets,
@@ -491,7 +492,8 @@ kcore_status kcore_decompose_static(int64_t n, int64_t m, const int64_t* offsets
  * vertex count. One peel at level kprime - 1 on the bulk-synchronous kernel:
  * a scan takes every vertex whose degree is below kprime, and subround passes
  * remove the vertices whose decrement lands them below kprime. kprime <= 0
- * keeps every vertex. Input layout, workspace and errors as kcore_decompose
+ * keeps every vertex; mask_out holds intermediate counts until the call has
+ * finished on the device. Input layout, workspace and errors as kcore_decompose
  * (asynchronous on `stream`; kcore_sync_status reports device errors). */
 kcore_status kcore_core_mask(kcore_handle h, int64_t n, int64_t m, const int64_t* offsets, const int32_t* adj,
                              int32_t kprime, int32_t* mask_out, int64_t* size_out, kcore_stream_t stream);
