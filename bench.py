@@ -539,8 +539,8 @@ def run_gpu(args):
             "csr_build": {"ms": min(csr_ms), "algorithmic_bytes": csr_build_bytes(n, E, m),
                           "achieved_gbs": csr_build_bytes(n, E, m) / (min(csr_ms) / 1e3) / 1e9,
                           "frac": csr_build_bytes(n, E, m) / (min(csr_ms) / 1e3) / 1e9 / peak,
-                          "note": "timed apart from the decomposition (a stable LSD radix sort of "
-                                  "2E keys, then unique + emit)"},
+                          "note": "timed apart from the decomposition (stable LSD radix sorts of "
+                                  "one key per edge, then unique + emit)"},
             "ms_min": min(step_ms), "ms_mean": sum(step_ms) / len(step_ms),
             "parallelism": "replicas" if ws > 1 else "single GPU",
             "wall_s": wall,
